@@ -1362,6 +1362,7 @@ __global__ void k_chi_k(int nk, const double* __restrict__ kp, const T* __restri
 
 #include "adjoint.cuh"
 #include "tri.cuh"
+#include "tri_dense.cuh"
 #include "tri_adj.cuh"
 
 // ----------------------------------------------------------------------------- objects
@@ -1447,6 +1448,18 @@ struct sr_flow {
     DevBuf<uint4> tlat_rec;
     DevBuf<int4> tlat_items;
     int tlat_n_items = 0;
+    // TRI vertex flow with the dense lattice sum (trid::): tables, packed state, and the flag that
+    // sends a state with odd components to the general kernel (graded lattices)
+    trid::Tab td{};
+    trid::Choice<float> tdf;
+    trid::Choice<double> tdd;
+    bool td_on = false, td_graded = false;
+    DevBuf<int2> td_pack;
+    DevBuf<unsigned> td_fmap;
+    DevBuf<int> td_ent, td_run_pair, td_n_terms, td_terms, td_flag;
+    DevBuf<int2> td_runs;
+    DevBuf<float> Pf;
+    DevBuf<double> Pd;
 
     Tabs tabs() const {
         Tabs t;
@@ -1505,6 +1518,44 @@ static sr_status prof_end(sr_flow* f, int id, cudaEvent_t b) {
     return SR_OK;
 }
 
+// TRI vertex flow of the stored pairs pb .. pe - 1 for the state G_s (nodes already tabulated), on
+// stream st: the dense-contraction kernel where the lattice's tables fit it, else the general one.
+// A graded lattice launches both; the flag set while packing lets exactly one of them run.
+static void launch_gamma_tri(sr_flow* f, const double* G_s, const float* Gf_s, double* dG_o, int pb, int pe, cudaStream_t st) {
+    const Geo& g = f->g;
+    const Tabs tb = f->tabs();
+    const int blocks = (pe - pb) * g.N;
+    const int* use = nullptr;
+    if (f->td_on) {
+        const unsigned pblocks = (unsigned)std::min<long>((long)g.npair * g.N, 4096);
+        if (f->td_graded) {
+            use = f->td_flag.p;
+            cudaMemsetAsync(f->td_flag.p, 0, sizeof(int), st);
+        }
+        if (f->prec == SR_FP64) {
+            if (f->td_graded) trid::k_tri_pack<double, true><<<pblocks, 128, 0, st>>>(g, f->td, G_s, f->Pd.p, f->td_flag.p);
+            else trid::k_tri_pack<double, false><<<pblocks, 128, 0, st>>>(g, f->td, G_s, f->Pd.p, nullptr);
+            f->tdd.fn<<<blocks, f->tdd.threads, f->tdd.smem, st>>>(g, tb, f->td, f->w.p, f->Pd.p, f->nx.p, f->nW.p, f->ncount.p,
+                                                                   dG_o, pb, use, 0);
+        } else {
+            if (f->td_graded) {
+                trid::k_tri_pack<float, true><<<pblocks, 128, 0, st>>>(g, f->td, G_s, f->Pf.p, f->td_flag.p);
+                trid::k_shadow_if<<<1024, 256, 0, st>>>(g.nent, G_s, f->Gf.p, f->td_flag.p);
+            } else {
+                trid::k_tri_pack<float, false><<<pblocks, 128, 0, st>>>(g, f->td, G_s, f->Pf.p, nullptr);
+            }
+            f->tdf.fn<<<blocks, f->tdf.threads, f->tdf.smem, st>>>(g, tb, f->td, f->w.p, f->Pf.p, f->nx.p, f->nW.p, f->ncount.p,
+                                                                   dG_o, pb, use, 0);
+        }
+        if (!f->td_graded) return;
+    }
+    const TabsT tt = f->tabs_tri();
+    if (f->prec == SR_FP64)
+        k_gamma_rhs_tri<double><<<blocks, kThreads, f->smem_rhs, st>>>(g, tb, tt, f->w.p, G_s, f->nx.p, f->nW.p, f->ncount.p, dG_o, pb, use);
+    else
+        k_gamma_rhs_tri<float><<<blocks, kThreads, f->smem_rhs, st>>>(g, tb, tt, f->w.p, Gf_s, f->nx.p, f->nW.p, f->ncount.p, dG_o, pb, use);
+}
+
 // Right-hand side at cutoff lam for the state (gam_s, G_s [, Gf_s]) into (dgam_o, dG_o).
 static sr_status run_rhs(sr_flow* f, double lam, const double* gam_s, const double* G_s, const float* Gf_s,
                          double* dgam_o, double* dG_o, int pb = 0, int pe = -1) {
@@ -1533,7 +1584,7 @@ static sr_status run_rhs(sr_flow* f, double lam, const double* gam_s, const doub
         if (sr_status s = prof_begin(f, 2, &e0)) return s;
         if (g.nc == 16)
             k_gamma_rhs_tri<DualT><<<blocks, kThreads, f->smem_rhs, f->stream>>>(g, tb, f->tabs_tri(), f->w.p, Gd, f->nx.p, nW,
-                                                                                   f->ncount.p, dGo, pb);
+                                                                                   f->ncount.p, dGo, pb, nullptr);
         else if (g.nc == 2)
             k_gamma_rhs<DualT, 2><<<blocks, kThreads, f->smem_rhs, f->stream>>>(g, tb, f->w.p, Gd, f->nx.p, nW, f->ncount.p, dGo, pb);
         else
@@ -1554,10 +1605,7 @@ static sr_status run_rhs(sr_flow* f, double lam, const double* gam_s, const doub
                                                                f->ncount.p, nullptr);
         if (sr_status s = prof_end(f, 1, e0)) return s;
         if (sr_status s = prof_begin(f, 2, &e0)) return s;
-        if (f->prec == SR_FP64)
-            k_gamma_rhs_tri<double><<<blocks, kThreads, f->smem_rhs, f->stream>>>(g, tb, tt, f->w.p, G_s, f->nx.p, f->nW.p, f->ncount.p, dG_o, pb);
-        else
-            k_gamma_rhs_tri<float><<<blocks, kThreads, f->smem_rhs, f->stream>>>(g, tb, tt, f->w.p, Gf_s, f->nx.p, f->nW.p, f->ncount.p, dG_o, pb);
+        launch_gamma_tri(f, G_s, Gf_s, dG_o, pb, pe, f->stream);
         if (sr_status s = prof_end(f, 2, e0)) return s;
         CK(cudaGetLastError());
         f->n_rhs++;
@@ -1603,6 +1651,7 @@ static sr_status run_rhs(sr_flow* f, double lam, const double* gam_s, const doub
 static sr_status refresh_shadow(sr_flow* f, const double* G_s, float* Gf_s) {
     if (f->prec != SR_FP32_MIXED) return SR_OK;
     if (f->g.nc == 16) {
+        if (f->td_on) return SR_OK;   // packed with the vertex launch
         const long n = f->g.nent;
         k_shadow_tri<<<(unsigned)((n + 255) / 256), 256, 0, f->stream>>>(n, G_s, Gf_s);
         CK(cudaGetLastError());
@@ -1914,13 +1963,52 @@ static sr_status flow_create(const sr_lattice* lat, int n_freq, const double* fr
         CK(f->chi_r16.upload(cr.data(), cr.size(), st));
         CK(f->chi_m16.upload(cm.data(), cm.size(), st));
         f->nprod = (int)(64 * P);   // products of the lattice sum per node (reported)
+        trid::Plan pl;
+        const long nrow = (long)g.npair * g.N;
+        // (packed offsets reach 2 nent; the two rows of a triple need 31-bit addressing)
+        if (!f->ntan && 2 * g.nent < (1L << 31) && trid::build_plan(lat, &pl)) {
+            bool on;
+            if (precision == SR_FP64) {
+                f->tdd = pl.graded ? trid::choose<double, true>(g.N, Ns, pl.nk, (int)pl.runs.size()) : trid::choose<double, false>(g.N, Ns, pl.nk, (int)pl.runs.size());
+                on = f->tdd.fn != nullptr;
+                if (on) CK(ensure_smem((const void*)f->tdd.fn, f->tdd.smem));
+            } else {
+                f->tdf = pl.graded ? trid::choose<float, true>(g.N, Ns, pl.nk, (int)pl.runs.size()) : trid::choose<float, false>(g.N, Ns, pl.nk, (int)pl.runs.size());
+                on = f->tdf.fn != nullptr;
+                if (on) CK(ensure_smem((const void*)f->tdf.fn, f->tdf.smem));
+            }
+            if (on) {
+                f->td_on = true;
+                f->td_graded = pl.graded;
+                CK(f->td_pack.upload(pl.pack.data(), pl.pack.size(), st));
+                CK(f->td_fmap.upload(pl.fmap.data(), pl.fmap.size(), st));
+                CK(f->td_ent.upload(pl.ent.data(), pl.ent.size(), st));
+                CK(f->td_runs.upload(pl.runs.data(), pl.runs.size(), st));
+                CK(f->td_run_pair.upload(pl.run_pair.data(), pl.run_pair.size(), st));
+                CK(f->td_n_terms.upload(pl.n_terms.data(), pl.n_terms.size(), st));
+                CK(f->td_terms.upload(pl.terms.data(), pl.terms.size(), st));
+                CK(f->td_flag.alloc(1));
+                trid::Tab& td = f->td;
+                td.pack = f->td_pack.p; td.fmap = f->td_fmap.p; td.ent = f->td_ent.p; td.runs = f->td_runs.p;
+                td.run_pair = f->td_run_pair.p; td.n_terms = f->td_n_terms.p; td.terms = f->td_terms.p;
+                td.n_runs = (int)pl.runs.size(); td.nk = pl.nk;
+                for (int k = 0; k < trid::kMaxPairs; ++k) td.kap[k] = pl.kap[k];
+                for (int k = 0; k < 4; ++k) td.spin[k] = pl.spin[k];
+                td.nrow = (int)nrow;
+                const unsigned long long half = (unsigned long long)(pl.graded ? Ns : 2 * Ns);
+                td.div_half = half > 1 ? (unsigned)((0x100000000ULL + half - 1) / half) : 0u;
+                const size_t np = (size_t)g.nent * (pl.graded ? 1 : 2);
+                if (precision == SR_FP64) CK(f->Pd.alloc(np));
+                else CK(f->Pf.alloc(np));
+            }
+        }
     }
     // state
     CK(f->gam.alloc((size_t)g.N * ts));
     CK(f->G.alloc((size_t)g.nent * ts));
     CK(f->dgam.alloc((size_t)g.N * ts));
     CK(f->dG.alloc((size_t)g.nent * ts));
-    if (precision == SR_FP32_MIXED) CK(f->Gf.alloc(g.nc == 16 ? (size_t)g.nent : (size_t)g.nentp * (f->has_swap ? 2 : 1)));
+    if (precision == SR_FP32_MIXED && !(f->td_on && !f->td_graded)) CK(f->Gf.alloc(g.nc == 16 ? (size_t)g.nent : (size_t)g.nentp * (f->has_swap ? 2 : 1)));
     CK(f->nx.alloc((size_t)3 * g.N * g.nmax));
     CK(f->nW.alloc((size_t)3 * g.N * g.nmax * ts));
     CK(f->nWf.alloc((size_t)3 * g.N * g.nmax));
@@ -2591,6 +2679,8 @@ struct BInst {
     int kind;       // 0 SU2 dense, 1 SU2 product list, 2 XYZ, 3 TRI
     int with_swap;
     int qb_own;     // SU2 dense: node block of the instance's own kernel (k_gamma_rhs_su2f)
+    sr_flow* flow;  // the instance (host)
+    int copy_f32;   // TRI: the FP32 copy is kept up to date (else the vertex launch packs the state)
 };
 
 __global__ void k_sigma_b(const BInst* __restrict__ I, const double* __restrict__ lams, const int* __restrict__ step) {
@@ -2738,7 +2828,8 @@ __global__ void k_shadow_b(const BInst* __restrict__ I) {
     const long stride = (long)gridDim.x * blockDim.x;
     if (B.kind == 3) {
         // TRI: FP32 copy of the state in its own layout
-        for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < g.nent; i += stride) B.Gf[i] = (float)B.G[i];
+        if (B.copy_f32)
+            for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < g.nent; i += stride) B.Gf[i] = (float)B.G[i];
         return;
     }
     for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < g.nentp; i += stride) {
@@ -2824,7 +2915,7 @@ static void launch_class(sr_batch* b, int k, cudaStream_t st) {
             else if (c.kind == 1)
                 k_gamma_rhs_f32<2, false><<<blocks, kThreads, sm, st>>>(B.g, B.tb, B.Gf, B.Gs, B.nxf, B.nWf, B.ncount, B.dG, 0);
             else if (c.kind == 3)
-                k_gamma_rhs_tri<float><<<blocks, kThreads, sm, st>>>(B.g, B.tb, B.tt, B.tb.w, B.Gf, B.nx, B.nW, B.ncount, B.dG, 0);
+                launch_gamma_tri(B.flow, B.G, B.Gf, B.dG, 0, B.g.npair, st);
             else
                 k_gamma_rhs_f32<4, false><<<blocks, kThreads, sm, st>>>(B.g, B.tb, B.Gf, B.Gs, B.nxf, B.nWf, B.ncount, B.dG, 0);
         }
@@ -3110,6 +3201,8 @@ extern "C" sr_status sr_batch_create(int n, sr_flow* const* flows, sr_batch** ou
         B.kind = kind[k];
         B.with_swap = f->has_swap ? 1 : 0;
         B.qb_own = f->su2f_qb;
+        B.flow = f;
+        B.copy_f32 = f->td_on ? 0 : 1;
         if (kind[k] == 0) B.qc = f->su2f_qb;
         unit += (long)f->g.npair * f->g.N;
         b->inst.push_back(B);

@@ -247,7 +247,9 @@ template <typename R>
 __global__ void __launch_bounds__(kThreads) k_gamma_rhs_tri(Geo g, Tabs tb, TabsT tt, const double* __restrict__ w,
                                                             const R* __restrict__ G, const double* __restrict__ nx,
                                                             const TriOut<R>* __restrict__ nW, const int* __restrict__ ncount,
-                                                            TriOut<R>* __restrict__ dG, int p0) {
+                                                            TriOut<R>* __restrict__ dG, int p0,
+                                                            const int* __restrict__ use) {
+    if (use && *use == 0) return;   // the graded form (tri_dense.cuh) serves this state
     using D = typename WeightOf<R>::type;                 // descriptor weights
     constexpr bool kFold = std::is_same<D, R>::value;     // node weights folded into the corner weights
     constexpr bool kF32 = std::is_same<R, float>::value;
