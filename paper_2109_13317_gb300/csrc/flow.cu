@@ -1184,8 +1184,6 @@ __global__ void __launch_bounds__(kThreads) k_gamma_rhs_f32_tc(Geo g, Tabs tb, c
     if (threadIdx.x < 32) tc::tmem_dealloc(tcs.tmem, ncols);
 }
 
-#include "su2f.cuh"
-
 // FP32 shadow of the state in the padded layout, and (with_swap) the exchanged copy in which
 // entry (c, r) holds the stored value of the pair (rep_r, ref): component perm(c) of site
 // swap_r[r].  Padding sites are zero.
@@ -1361,6 +1359,7 @@ __global__ void k_chi_k(int nk, const double* __restrict__ kp, const T* __restri
 }  // namespace
 
 #include "adjoint.cuh"
+#include "pair.cuh"
 #include "tri.cuh"
 #include "tri_dense.cuh"
 #include "tri_adj.cuh"
@@ -1409,8 +1408,6 @@ struct sr_flow {
     DevBuf<int> dgath_idx;
     bool has_swap = false, dense = false;
     bool use_tc = false;          // FP32-mixed SU2: lattice sum on the tensor cores
-    size_t smem_su2f = 0;         // FP32-mixed SU2 kernel (k_gamma_rhs_su2f): dynamic shared memory,
-    int su2f_qb = 0;              // its integration nodes per block (0: the kernel is not used)
     size_t smem_tc = 0;           // dynamic shared memory of the tensor-core kernel
     int tc_grid = 0;              // its persistent grid (SMs x resident CTAs)
     int tc_occ_api = 0;           // the runtime's occupancy figure for it (reported only)
@@ -1448,6 +1445,14 @@ struct sr_flow {
     DevBuf<uint4> tlat_rec;
     DevBuf<int4> tlat_items;
     int tlat_n_items = 0;
+    // SU2 / XYZ vertex flow (pairk::): tables, kernel variant and packed state
+    bool pk_on = false;
+    pairk::Tab pk{};
+    int pk_variant = -1, pk_threads = 0;
+    size_t pk_smem = 0;
+    DevBuf<int> pk_terms, pk_n_terms, pk_kap;
+    DevBuf<int2> pk_prod;
+    DevBuf<double> pk_mult;
     // TRI vertex flow with the dense lattice sum (trid::): tables, packed state, and the flag that
     // sends a state with odd components to the general kernel (graded lattices)
     trid::Tab td{};
@@ -1516,6 +1521,32 @@ static sr_status prof_end(sr_flow* f, int id, cudaEvent_t b) {
     CK(cudaEventRecord(e, f->stream));
     f->ev[id].push_back({b, e});
     return SR_OK;
+}
+
+// SU2 / XYZ: pack the state G_s for the vertex kernel.
+static void launch_pack_pair(sr_flow* f, const double* G_s, cudaStream_t st) {
+    const Geo& g = f->g;
+    const Tabs tb = f->tabs();
+    const unsigned nb = (unsigned)std::min<long>(((long)f->pk.nrow * g.Ns + 255) / 256, 8192);
+    if (f->prec == SR_FP64) {
+        if (g.nc == 2) pairk::k_pair_pack<double, 2><<<nb, 256, 0, st>>>(g, tb, f->pk, G_s, f->Pd.p);
+        else pairk::k_pair_pack<double, 4><<<nb, 256, 0, st>>>(g, tb, f->pk, G_s, f->Pd.p);
+    } else {
+        if (g.nc == 2) pairk::k_pair_pack<float, 2><<<nb, 256, 0, st>>>(g, tb, f->pk, G_s, f->Pf.p);
+        else pairk::k_pair_pack<float, 4><<<nb, 256, 0, st>>>(g, tb, f->pk, G_s, f->Pf.p);
+    }
+}
+
+// SU2 / XYZ: vertex flow of the stored pairs pb .. pe - 1 from the packed state.
+static void launch_gamma_pair(sr_flow* f, double* dG_o, int pb, int pe, cudaStream_t st) {
+    const Tabs tb = f->tabs();
+    const int blocks = (pe - pb) * f->g.N;
+    if (f->prec == SR_FP64)
+        pairk::kernel_f64(f->pk_variant)<<<blocks, f->pk_threads, f->pk_smem, st>>>(f->g, tb, f->pk, f->Pd.p, f->nx.p, f->nW.p,
+                                                                                     f->ncount.p, dG_o, pb);
+    else
+        pairk::kernel_f32(f->pk_variant)<<<blocks, f->pk_threads, f->pk_smem, st>>>(f->g, tb, f->pk, f->Pf.p, f->nxf.p, f->nWf.p,
+                                                                                     f->ncount.p, dG_o, pb);
 }
 
 // TRI vertex flow of the stored pairs pb .. pe - 1 for the state G_s (nodes already tabulated), on
@@ -1619,22 +1650,21 @@ static sr_status run_rhs(sr_flow* f, double lam, const double* gam_s, const doub
                                                            f->ncount.p, f->prec == SR_FP32_MIXED ? f->nxf.p : nullptr);
     if (sr_status s = prof_end(f, 1, e0)) return s;
     if (sr_status s = prof_begin(f, 2, &e0)) return s;
-    if (f->prec == SR_FP64) {
+    if (f->pk_on && !f->use_tc) {
+        launch_pack_pair(f, G_s, f->stream);
+        launch_gamma_pair(f, dG_o, pb, pe, f->stream);
+    } else if (f->prec == SR_FP64) {
         if (g.nc == 2)
             k_gamma_rhs<double, 2><<<blocks, kThreads, f->smem_rhs, f->stream>>>(g, tb, f->w.p, G_s, f->nx.p, f->nW.p, f->ncount.p, dG_o, pb);
         else
             k_gamma_rhs<double, 4><<<blocks, kThreads, f->smem_rhs, f->stream>>>(g, tb, f->w.p, G_s, f->nx.p, f->nW.p, f->ncount.p, dG_o, pb);
     } else {
         const float* Gs = f->has_swap ? Gf_s + g.nentp : Gf_s;
+        if (f->pk_on)   // the tensor-core path of a flow whose own kernel packs the state
+            k_shadow<<<(unsigned)((g.nentp + 255) / 256), 256, 0, f->stream>>>(g, tb, G_s, f->Gf.p, f->has_swap ? 1 : 0);
         if (g.nc == 2 && f->dense && f->use_tc)
             k_gamma_rhs_f32_tc<<<std::min(blocks, f->tc_grid), kThreads, f->smem_tc, f->stream>>>(g, tb, Gf_s, Gs, f->nxf.p, f->nWf.p, f->ncount.p, dG_o,
                                                                             f->tcfail.p, (long)pb * g.N, (long)pe * g.N);
-        else if (g.nc == 2 && f->dense && f->su2f_qb > 0 && su2f::cache_for(g.nsp))
-            k_gamma_rhs_su2f<true><<<blocks, su2f::threads_for(g.nsp), f->smem_su2f, f->stream>>>(
-                g, tb, Gf_s, f->has_swap ? (int)g.nentp : 0, f->nxf.p, f->nWf.p, f->ncount.p, dG_o, f->su2f_qb, pb);
-        else if (g.nc == 2 && f->dense && f->su2f_qb > 0)
-            k_gamma_rhs_su2f<false><<<blocks, su2f::threads_for(g.nsp), f->smem_su2f, f->stream>>>(
-                g, tb, Gf_s, f->has_swap ? (int)g.nentp : 0, f->nxf.p, f->nWf.p, f->ncount.p, dG_o, f->su2f_qb, pb);
         else if (g.nc == 2 && f->dense)
             k_gamma_rhs_f32<2, true><<<blocks, kThreads, f->smem_rhs, f->stream>>>(g, tb, Gf_s, Gs, f->nxf.p, f->nWf.p, f->ncount.p, dG_o, pb);
         else if (g.nc == 2)
@@ -1657,6 +1687,7 @@ static sr_status refresh_shadow(sr_flow* f, const double* G_s, float* Gf_s) {
         CK(cudaGetLastError());
         return SR_OK;
     }
+    if (f->pk_on) return SR_OK;   // packed with the vertex launch (tensor cores: copied there)
     long n = f->g.nentp;
     k_shadow<<<(unsigned)((n + 255) / 256), 256, 0, f->stream>>>(f->g, f->tabs(), G_s, Gf_s, f->has_swap ? 1 : 0);
     CK(cudaGetLastError());
@@ -1847,6 +1878,34 @@ static sr_status flow_create(const sr_lattice* lat, int n_freq, const double* fr
             dg[k] = ca * nsp * nsp + ra * nsp + rb;
         }
         CK(f->dgath_idx.upload(dg.data(), dg.size(), f->stream));
+        pairk::Plan pl;
+        if (!f->ntan && pairk::build_plan(lat, n_freq, precision != SR_FP64, f->has_swap, prods, goff, gidx, &pl)) {
+            f->pk_on = true;
+            f->pk = pl.td;
+            f->pk_variant = pl.variant;
+            f->pk_threads = pl.threads;
+            f->pk_smem = pl.smem;
+            CK(f->pk_terms.upload(pl.terms.data(), pl.terms.size(), f->stream));
+            CK(f->pk_n_terms.upload(pl.n_terms.data(), pl.n_terms.size(), f->stream));
+            CK(f->pk_prod.upload(pl.prod.data(), pl.prod.size(), f->stream));
+            CK(f->pk_kap.upload(pl.kap.data(), pl.kap.size(), f->stream));
+            CK(f->pk_mult.upload(pl.mult.data(), pl.mult.size(), f->stream));
+            f->pk.kap = f->pk_kap.p;
+            f->pk.mult = f->pk_mult.p;
+            f->pk.terms = f->pk_terms.p;
+            f->pk.n_terms = f->pk_n_terms.p;
+            f->pk.prod = f->pk_prod.p;
+            const size_t np = (size_t)pl.size;
+            if (precision == SR_FP64) {
+                CK(f->Pd.alloc(np));
+                CK(cudaMemsetAsync(f->Pd.p, 0, sizeof(double) * np, f->stream));   // padding stays zero
+                CK(ensure_smem((const void*)pairk::kernel_f64(pl.variant), pl.smem));
+            } else {
+                CK(f->Pf.alloc(np));
+                CK(cudaMemsetAsync(f->Pf.p, 0, sizeof(float) * np, f->stream));
+                CK(ensure_smem((const void*)pairk::kernel_f32(pl.variant), pl.smem));
+            }
+        }
     }
     std::vector<double> ih(n_freq - 1);
     for (int i = 0; i + 1 < n_freq; ++i) ih[i] = 1.0 / (freq_pos[i + 1] - freq_pos[i]);
@@ -2008,7 +2067,8 @@ static sr_status flow_create(const sr_lattice* lat, int n_freq, const double* fr
     CK(f->G.alloc((size_t)g.nent * ts));
     CK(f->dgam.alloc((size_t)g.N * ts));
     CK(f->dG.alloc((size_t)g.nent * ts));
-    if (precision == SR_FP32_MIXED && !(f->td_on && !f->td_graded)) CK(f->Gf.alloc(g.nc == 16 ? (size_t)g.nent : (size_t)g.nentp * (f->has_swap ? 2 : 1)));
+    if (precision == SR_FP32_MIXED && !(f->td_on && !f->td_graded) && !f->pk_on)
+        CK(f->Gf.alloc(g.nc == 16 ? (size_t)g.nent : (size_t)g.nentp * (f->has_swap ? 2 : 1)));
     CK(f->nx.alloc((size_t)3 * g.N * g.nmax));
     CK(f->nW.alloc((size_t)3 * g.N * g.nmax * ts));
     CK(f->nWf.alloc((size_t)3 * g.N * g.nmax));
@@ -2047,19 +2107,6 @@ static sr_status flow_create(const sr_lattice* lat, int n_freq, const double* fr
         CK(ensure_smem((const void*)k_gamma_rhs<double, 4>, f->smem_rhs));
     } else {
         CK(ensure_smem((const void*)k_gamma_rhs_f32<2, true>, f->smem_rhs));
-        if (g.nc == 2 && f->dense && g.nsp / 2 <= su2f::kThreadsS) {
-            // FP32-mixed SU2 kernel: the largest node block (64, 32, 16) whose shared memory
-            // leaves room for the resident CTAs its registers allow, else the smallest that fits
-            const int nth = su2f::threads_for(g.nsp);
-            const int ctas = (su2f::cache_for(g.nsp) ? su2f::kMinCtasCached : su2f::kMinCtas) * su2f::kThreadsS / nth;
-            for (int qb : {64, 32, 16}) {
-                const size_t b = su2f::layout(g.N, g.Ns, g.nsp, qb, nth).total;
-                if (b <= 227 * 1024 / ctas || (qb == 16 && b <= 227 * 1024)) { f->su2f_qb = qb; f->smem_su2f = b; break; }
-            }
-            if (f->su2f_qb > 0)
-                CK(ensure_smem(su2f::cache_for(g.nsp) ? (const void*)k_gamma_rhs_su2f<true> : (const void*)k_gamma_rhs_su2f<false>,
-                               f->smem_su2f));
-        }
         CK(ensure_smem((const void*)k_gamma_rhs_f32<2, false>, f->smem_rhs));
         CK(ensure_smem((const void*)k_gamma_rhs_f32<4, false>, f->smem_rhs));
         if (tc_ok) {
@@ -2103,6 +2150,13 @@ extern "C" sr_status sr_flow_set_tensor_cores(sr_flow* f, int on) {
     if (!f) return fail(SR_EINVAL, "null flow");
     if (on && !(f->prec == SR_FP32_MIXED && tc_supported(f->g.nc, f->g.nsp, f->dense)))
         return fail(SR_EUNSUPPORTED, "tensor-core lattice sum needs an FP32-mixed SU2 flow with at most 64 padded sites");
+    if (on && !f->Gf.p) {   // its copy of the state (a flow on the packed state has none)
+        if (f->Gf.alloc((size_t)f->g.nentp * (f->has_swap ? 2 : 1)) != cudaSuccess) {
+            cudaGetLastError();
+            f->Gf.p = nullptr;
+            return fail(SR_ENOMEM, "no device memory for the tensor-core path's copy of the state");
+        }
+    }
     f->use_tc = on != 0;
     return SR_OK;
 }
@@ -2676,9 +2730,10 @@ struct BInst {
     int* ncount;
     long unit0;     // first work unit (stored triple) of this instance
     int qc;         // integration nodes per shared-memory block
-    int kind;       // 0 SU2 dense, 1 SU2 product list, 2 XYZ, 3 TRI
+    int kind;       // 0 SU2 / XYZ on the packed state (pairk), 2 XYZ general kernel, 3 TRI
     int with_swap;
-    int qb_own;     // SU2 dense: node block of the instance's own kernel (k_gamma_rhs_su2f)
+    pairk::Tab pk;  // kind 0: tables and packed state
+    float* P;
     sr_flow* flow;  // the instance (host)
     int copy_f32;   // TRI: the FP32 copy is kept up to date (else the vertex launch packs the state)
 };
@@ -2731,22 +2786,21 @@ __global__ void __launch_bounds__(kThreads, 7) k_gamma_persistent(const BInst* _
             __syncthreads();
         }
         const long local = u - B.unit0;
-        const Geo g = B.g;   // locals: see k_gamma_persistent_su2f
+        const Geo g = B.g;   // locals: see k_gamma_persistent_pair
         const Tabs tb = B.tb;
         const int p = (int)(local / g.N), ti = (int)(local % g.N);
         gamma_rhs_f32_triple<NC, DENSE>(g, tb, B.Gf, B.Gs, B.nxf, B.nWf, B.ncount, B.dG, p, ti, smem, B.qc);
     }
 }
 
-// SU2 instances (dense lattice sum) in one persistent kernel over the per-triple function of
-// k_gamma_rhs_su2f: CTAs take `chunk` consecutive units per atomic step (consecutive units
-// mostly belong to one instance, whose tables are staged once), with the register budget of
-// the instances' own kernel.  CACHE: the corner-row cache of k_gamma_rhs_su2f<true> (classes of
-// wide rows).
-template <bool CACHE>
-__global__ void __launch_bounds__(su2f::kThreadsS, CACHE ? su2f::kMinCtasCached : su2f::kMinCtas) k_gamma_persistent_su2f(const BInst* __restrict__ I, int i_begin, int i_end,
-                                                                    long u_begin, long u_end,
-                                                                    unsigned long long* __restrict__ counter, int chunk) {
+// SU2 and XYZ instances in one persistent kernel over the per-triple function of k_gamma_rhs_pair:
+// CTAs take `chunk` consecutive units per atomic step (consecutive units mostly belong to one
+// instance, whose tables are staged once), with the variant, CTA size and register budget of the
+// instances' own kernel.
+template <int NC, int TM, int TN, int NT, int MAXT, int MINB>
+__global__ void __launch_bounds__(MAXT, MINB) k_gamma_persistent_pair(const BInst* __restrict__ I, int i_begin, int i_end,
+                                                                      long u_begin, long u_end,
+                                                                      unsigned long long* __restrict__ counter, int chunk) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ long unit_sh;
     __shared__ __align__(16) BInst B;   // the current unit's instance
@@ -2785,22 +2839,30 @@ __global__ void __launch_bounds__(su2f::kThreadsS, CACHE ? su2f::kMinCtasCached 
             // shared memory would otherwise force re-reads of every field from the shared copy
             const Geo g = B.g;
             const Tabs tb = B.tb;
-            su2f::triple<CACHE>(g, tb, B.Gf, B.with_swap ? (int)g.nentp : 0, B.nxf, B.nWf, B.ncount, B.dG,
-                                (int)(local / g.N), (int)(local % g.N), smem, B.qc);
+            const pairk::Tab td = B.pk;
+            pairk::triple<float, NC, TM, TN, NT>(g, tb, td, B.P, B.nxf, B.nWf, B.ncount, B.dG, (int)(local / g.N),
+                                                 (int)(local % g.N), smem);
         }
     }
 }
 
-// Units per atomic step of the SU2 persistent kernel.
+// Units per atomic step of the pair persistent kernel.
 constexpr int kUnitChunk = 4;
 
-// Persistent kernel of an instance kind (0: SU2 dense lattice sum, 1: SU2 product list, 2: XYZ;
-// TRI instances, kind 3, always run their own kernels); every size class holds instances of
-// one kind.
-static const void* persistent_fn(int kind, bool cache = false) {
-    if (kind == 0) return cache ? (const void*)k_gamma_persistent_su2f<true> : (const void*)k_gamma_persistent_su2f<false>;
-    if (kind == 1) return (const void*)k_gamma_persistent<2, false>;
-    return (const void*)k_gamma_persistent<4, false>;
+using PersistentPair = void (*)(const BInst*, int, int, long, long, unsigned long long*, int);
+static PersistentPair persistent_pair(int variant) {
+#define PAIR_CASE(id, NC, TM, TN, NT, MAXT, MINB, PAD) \
+    case id: return k_gamma_persistent_pair<NC, TM, TN, NT, MAXT, MINB>;
+    switch (variant) { PAIR_F32_VARIANTS(PAIR_CASE) }
+#undef PAIR_CASE
+    return nullptr;
+}
+
+// Persistent kernel of an instance kind (0: packed-state kernel in the given variant, 2: XYZ general
+// kernel; TRI instances, kind 3, always run their own kernels); every size class holds instances of
+// one kind and variant.
+static const void* persistent_fn(int kind, int variant) {
+    return kind == 0 ? (const void*)persistent_pair(variant) : (const void*)k_gamma_persistent<4, false>;
 }
 
 // Euler update of every instance (y <- y - (Lambda_k - Lambda_k+1) f) and its FP32 shadow.
@@ -2826,6 +2888,7 @@ __global__ void k_shadow_b(const BInst* __restrict__ I) {
     const Geo& g = B.g;
     const int rowp = g.nc * g.nsp;
     const long stride = (long)gridDim.x * blockDim.x;
+    if (B.kind == 0) return;   // packed before the vertex launch
     if (B.kind == 3) {
         // TRI: FP32 copy of the state in its own layout
         if (B.copy_f32)
@@ -2847,6 +2910,20 @@ __global__ void k_shadow_b(const BInst* __restrict__ I) {
     }
 }
 
+// Packed state of the instances whose vertex kernel reads it.
+__global__ void k_pack_b(const BInst* __restrict__ I) {
+    const BInst& B = I[blockIdx.y];
+    if (B.kind != 0) return;
+    const Geo g = B.g;
+    const Tabs tb = B.tb;
+    const pairk::Tab td = B.pk;
+    const long n = (long)td.nrow * g.Ns;
+    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
+        if (g.nc == 2) pairk::pack_site<float, 2>(g, tb, td, B.G, B.P, i);
+        else pairk::pack_site<float, 4>(g, tb, td, B.G, B.P, i);
+    }
+}
+
 __global__ void k_advance(int* __restrict__ step, unsigned long long* __restrict__ counter, int ncounter) {
     *step += 1;
     for (int i = 0; i < ncounter; ++i) counter[i] = 0ULL;
@@ -2861,7 +2938,7 @@ struct BClass {
     size_t smem;
     int occ, ctas, qc;
     int threads;          // CTA size of the class's persistent kernel
-    bool cache;           // SU2: the corner-row cache (k_gamma_rhs_su2f<true>) for wide rows
+    int variant;          // kind 0: kernel variant of its instances
     double ms;            // autotuned vertex-flow time of the class
     bool per_inst;        // the instances' own vertex kernels, one launch each, instead of the
                           // class's persistent kernel
@@ -2906,14 +2983,7 @@ static void launch_class(sr_batch* b, int k, cudaStream_t st) {
             const BInst& B = b->inst[i];
             const unsigned blocks = (unsigned)(B.g.npair * B.g.N);
             const size_t sm = b->inst_smem[i];
-            if (c.kind == 0 && su2f::cache_for(B.g.nsp))
-                k_gamma_rhs_su2f<true><<<blocks, su2f::threads_for(B.g.nsp), sm, st>>>(
-                    B.g, B.tb, B.Gf, B.with_swap ? (int)B.g.nentp : 0, B.nxf, B.nWf, B.ncount, B.dG, B.qb_own, 0);
-            else if (c.kind == 0)
-                k_gamma_rhs_su2f<false><<<blocks, su2f::threads_for(B.g.nsp), sm, st>>>(
-                    B.g, B.tb, B.Gf, B.with_swap ? (int)B.g.nentp : 0, B.nxf, B.nWf, B.ncount, B.dG, B.qb_own, 0);
-            else if (c.kind == 1)
-                k_gamma_rhs_f32<2, false><<<blocks, kThreads, sm, st>>>(B.g, B.tb, B.Gf, B.Gs, B.nxf, B.nWf, B.ncount, B.dG, 0);
+            if (c.kind == 0) launch_gamma_pair(B.flow, B.dG, 0, B.g.npair, st);
             else if (c.kind == 3)
                 launch_gamma_tri(B.flow, B.G, B.Gf, B.dG, 0, B.g.npair, st);
             else
@@ -2924,10 +2994,7 @@ static void launch_class(sr_batch* b, int k, cudaStream_t st) {
     const dim3 grid(b->nsm * c.ctas);
     unsigned long long* ctr = b->counter.p + k;
     if (c.kind == 0)
-        (c.cache ? k_gamma_persistent_su2f<true> : k_gamma_persistent_su2f<false>)<<<grid, c.threads, c.smem, st>>>(
-            b->dinst.p, c.i_begin, c.i_end, c.u_begin, c.u_end, ctr, kUnitChunk);
-    else if (c.kind == 1)
-        k_gamma_persistent<2, false><<<grid, kThreads, c.smem, st>>>(b->dinst.p, c.i_begin, c.i_end, c.u_begin, c.u_end, ctr);
+        persistent_pair(c.variant)<<<grid, c.threads, c.smem, st>>>(b->dinst.p, c.i_begin, c.i_end, c.u_begin, c.u_end, ctr, kUnitChunk);
     else
         k_gamma_persistent<4, false><<<grid, kThreads, c.smem, st>>>(b->dinst.p, c.i_begin, c.i_end, c.u_begin, c.u_end, ctr);
 }
@@ -2951,6 +3018,14 @@ static sr_status launch_classes(sr_batch* b) {
     return SR_OK;
 }
 
+static void batch_pack(sr_batch* b) {
+    long most = 0;
+    for (const BInst& B : b->inst)
+        if (B.kind == 0) most = std::max(most, (long)B.pk.nrow * B.g.Ns);
+    if (most > 0)
+        k_pack_b<<<dim3((unsigned)std::min<long>((most + 255) / 256, 4 * b->nsm), (unsigned)b->inst.size()), 256, 0, b->stream>>>(b->dinst.p);
+}
+
 static sr_status batch_launch_step(sr_batch* b) {
     const int ni = (int)b->inst.size();
     int maxN = 0;
@@ -2958,6 +3033,7 @@ static sr_status batch_launch_step(sr_batch* b) {
     for (const BInst& B : b->inst) { maxN = std::max(maxN, B.g.N); maxent = std::max(maxent, B.g.nentp); }
     k_sigma_b<<<dim3(maxN, ni), 64, 0, b->stream>>>(b->dinst.p, b->lams.p, b->step.p);
     k_nodes_b<<<dim3(3 * maxN, ni), 128, 0, b->stream>>>(b->dinst.p, b->lams.p, b->step.p);
+    batch_pack(b);
     if (sr_status s = launch_classes(b)) return s;
     const int ub = (int)std::min<long>((maxent + 255) / 256, 4 * b->nsm);
     k_update_b<<<dim3(ub, ni), 256, 0, b->stream>>>(b->dinst.p, b->lams.p, b->step.p, b->flag.p);
@@ -3012,24 +3088,13 @@ static sr_status batch_tune(sr_batch* b) {
             total += ms;
             continue;
         }
-        // candidates (node block, shared memory, resident CTAs per SM): SU2 launches with the
-        // shared memory its node block needs, so small blocks raise the occupancy
+        // candidates (node block, shared memory, resident CTAs per SM); the packed-state kernel has
+        // one node block
         struct Cand { int qc; size_t smem; int occ; };
         std::vector<Cand> cand;
-        if (c.kind == 0) {
-            for (int qb : {16, 32, 64}) {
-                size_t need = 0;
-                for (int i = c.i_begin; i < c.i_end; ++i)
-                    need = std::max(need, su2f::layout(b->inst[i].g.N, b->inst[i].g.Ns, b->inst[i].g.nsp, qb, c.threads).total);
-                if (need > 227 * 1024) continue;
-                CK(ensure_smem(persistent_fn(c.kind, c.cache), need));
-                int occ = 0;
-                CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, persistent_fn(c.kind, c.cache), c.threads, need));
-                if (occ >= 1) cand.push_back({qb, need, occ});
-            }
-        } else {
+        if (c.kind == 0) cand.push_back({c.qc, c.smem, c.occ});
+        else
             for (int qb : qcs) cand.push_back({qb, c.smem, c.occ});
-        }
         if (cand.empty()) return fail(SR_EUNSUPPORTED, "size class %d: no node block fits the persistent kernel", k);
         double best = 1e300;
         int bq = c.qc, bc = c.ctas;
@@ -3133,31 +3198,21 @@ extern "C" sr_status sr_batch_create(int n, sr_flow* const* flows, sr_batch** ou
     std::vector<int> kind(n);
     for (int i = 0; i < n; ++i) {
         sr_flow* f = flows[i];
-        kind[i] = f->g.nc == 16 ? 3 : (f->g.nc == 4 ? 2 : (f->dense ? 0 : 1));
-        if (kind[i] == 0 && f->su2f_qb == 0)
+        kind[i] = f->g.nc == 16 ? 3 : (f->pk_on ? 0 : 2);
+        if (kind[i] == 2 && f->g.nc == 2)
             return fail(SR_EUNSUPPORTED, "flow %d: lattice too large for the batched SU2 kernel", i);
-        // SU2 dense: shared memory of the largest node block that fits (the tuner may pick it)
-        if (kind[i] == 0) {
-            const int nth = su2f::threads_for(f->g.nsp);
-            sm[i] = f->smem_su2f;
-            for (int qb : {64, 32}) {
-                const size_t bq = su2f::layout(f->g.N, f->g.Ns, f->g.nsp, qb, nth).total;
-                if (bq <= 227 * 1024 / 3) { sm[i] = std::max(sm[i], bq); break; }
-            }
-        } else if (kind[i] == 3) {
-            sm[i] = f->smem_rhs;
-        } else {
-            sm[i] = f32_smem_bytes(f->g.Ns, f->g.nsp, f->g.nc, f->nprod, f->dense);
-        }
+        if (kind[i] == 0) sm[i] = f->pk_smem;
+        else if (kind[i] == 3) sm[i] = f->smem_rhs;
+        else sm[i] = f32_smem_bytes(f->g.Ns, f->g.nsp, f->g.nc, f->nprod, f->dense);
     }
     std::vector<int> order(n);
     for (int i = 0; i < n; ++i) order[i] = i;
-    // SU2 instances whose own kernel is k_gamma_rhs_su2f<true> (wide rows) form classes of their
-    // own, so that every class's persistent kernel has its instances' CTA size and variant
-    auto wide = [&](int i) { return kind[i] == 0 && su2f::cache_for(flows[i]->g.nsp); };
+    // packed-state instances of different variants or CTA sizes form classes of their own, so that
+    // every class's persistent kernel has its instances' variant and CTA size
+    auto form = [&](int i) { return kind[i] == 0 ? flows[i]->pk_variant * 1024 + flows[i]->pk_threads : 0; };
     std::stable_sort(order.begin(), order.end(), [&](int a, int c) {
         if (kind[a] != kind[c]) return kind[a] < kind[c];
-        if (wide(a) != wide(c)) return wide(a);
+        if (form(a) != form(c)) return form(a) > form(c);
         if (sm[a] != sm[c]) return sm[a] > sm[c];
         return flows[a]->g.nent > flows[c]->g.nent;
     });
@@ -3168,22 +3223,22 @@ extern "C" sr_status sr_batch_create(int n, sr_flow* const* flows, sr_batch** ou
     for (int idx = 0; idx < n; ++idx) {
         const int k = order[idx];
         sr_flow* f = flows[k];
-        // a new class for a new kind or row width, or when the shared memory drops below 2/3 of
+        // a new class for a new kind or kernel form, or when the shared memory drops below 2/3 of
         // the class's largest
-        if (b->cls.empty() || b->cls.back().kind != kind[k] || b->cls.back().cache != wide(k) ||
+        if (b->cls.empty() || b->cls.back().kind != kind[k] || form(order[b->cls.back().i_begin]) != form(k) ||
             sm[k] * 3 < b->cls.back().smem * 2) {
             BClass c{};
             c.kind = kind[k];
-            c.i_begin = idx; c.u_begin = unit; c.smem = sm[k]; c.qc = kind[k] == 0 ? f->su2f_qb : kQF;
-            c.threads = kind[k] == 0 ? su2f::threads_for(f->g.nsp) : kThreads;
-            c.cache = kind[k] == 0 && su2f::cache_for(f->g.nsp);
+            c.i_begin = idx; c.u_begin = unit; c.smem = sm[k]; c.qc = kind[k] == 0 ? pairk::qrows<float>() : kQF;
+            c.threads = kind[k] == 0 ? f->pk_threads : kThreads;
+            c.variant = kind[k] == 0 ? f->pk_variant : -1;
             if (sm[k] > 227 * 1024) return fail(SR_EUNSUPPORTED, "instance needs %zu bytes of shared memory", sm[k]);
             if (c.kind == 3) {
                 c.occ = 1;   // no persistent kernel: the instances' own launches
                 c.per_inst = true;
             } else {
-                CK(ensure_smem(persistent_fn(c.kind, c.cache), sm[k]));
-                CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c.occ, persistent_fn(c.kind, c.cache), c.threads, sm[k]));
+                CK(ensure_smem(persistent_fn(c.kind, c.variant), sm[k]));
+                CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c.occ, persistent_fn(c.kind, c.variant), c.threads, sm[k]));
                 if (c.occ < 1) return fail(SR_EUNSUPPORTED, "persistent kernel cannot be resident with %zu bytes", sm[k]);
             }
             c.ctas = c.occ;
@@ -3200,13 +3255,14 @@ extern "C" sr_status sr_batch_create(int n, sr_flow* const* flows, sr_batch** ou
         B.qc = kQF;
         B.kind = kind[k];
         B.with_swap = f->has_swap ? 1 : 0;
-        B.qb_own = f->su2f_qb;
+        B.pk = f->pk;
+        B.P = f->Pf.p;
         B.flow = f;
         B.copy_f32 = f->td_on ? 0 : 1;
-        if (kind[k] == 0) B.qc = f->su2f_qb;
+        if (kind[k] == 0) B.qc = pairk::qrows<float>();
         unit += (long)f->g.npair * f->g.N;
         b->inst.push_back(B);
-        b->inst_smem.push_back(kind[k] == 0 ? f->smem_su2f : f->smem_rhs);   // TRI: k_gamma_rhs_tri<float>
+        b->inst_smem.push_back(f->smem_rhs);
         b->cls.back().i_end = idx + 1;
         b->cls.back().u_end = unit;
     }
@@ -3265,6 +3321,7 @@ extern "C" sr_status sr_batch_run(sr_batch* b, int n_lambda, const double* lambd
         CK(cudaMemcpyAsync(b->step.p, &mid, sizeof(int), cudaMemcpyHostToDevice, b->stream));
         k_sigma_b<<<dim3(maxN, ni), 64, 0, b->stream>>>(b->dinst.p, b->lams.p, b->step.p);
         k_nodes_b<<<dim3(3 * maxN, ni), 128, 0, b->stream>>>(b->dinst.p, b->lams.p, b->step.p);
+        batch_pack(b);
         CK(cudaGetLastError());
         if (sr_status s = batch_tune(b)) return s;
         // back to the first step, with the work counters the tuning launches consumed reset

@@ -271,7 +271,7 @@ k_gamma_rhs_trid(Geo g, Tabs tb, Tab td, const double* __restrict__ w, const R* 
                  const double* __restrict__ nW, const int* __restrict__ ncount, double* __restrict__ dG, int p0,
                  const int* __restrict__ use, int use_value) {
     if (use && (*use != 0) != (use_value != 0)) return;
-    constexpr int NCm = ncomp<GR>(), NM = nmu<GR>(), QB = qblock<R>(), NL = NM;
+    constexpr int NCm = ncomp<GR>(), NM = nmu<GR>(), QB = qblock<R>();
     extern __shared__ __align__(16) unsigned char smem[];
     const int tid = threadIdx.x, nth = blockDim.x, Ns = g.Ns;
     const int ld = row_ld<R, GR>(Ns), LM = NM * Ns, rowq = 4 * ld;   // one row (A or B) of a node: 4 kappa vectors
