@@ -548,13 +548,18 @@ k_gamma_rhs_trid(Geo g, Tabs tb, Tab td, const double* __restrict__ w, const R* 
         const int m = o / Ns, r = o - m * Ns;
         R a = R(0), l = R(0);
         for (int k = 0; k < NG; ++k) a += part[((size_t)k * Ns + r) * NCm + m];
+        // (four partial sums: independent loads, and a smaller rounding error of the long FP32 lists)
         const int nt = td.n_terms[r];
-#pragma unroll 4
-        for (int j = 0; j < nt; ++j) {
-            const int c = td.terms[(size_t)j * Ns * NCm + o];
-            const R v = src[c & 0x3fffffff];
-            l += (c >> 30) & 1 ? -v : v;
-        }
+        R lp[4] = {R(0), R(0), R(0), R(0)};
+        for (int j = 0; j < nt; j += 4)
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (j + i < nt) {
+                    const int c = td.terms[(size_t)(j + i) * Ns * NCm + o];
+                    const R v = src[c & 0x3fffffff];
+                    lp[i] += (c >> 30) & 1 ? -v : v;
+                }
+        l = (lp[0] + lp[1]) + (lp[2] + lp[3]);
         const int mu = mu_of(GR, m), nu = nu_of(GR, m);
         out[(td.spin[mu] * 4 + td.spin[nu]) * Ns + r] = (double)a - 2.0 * (double)l;
     }
