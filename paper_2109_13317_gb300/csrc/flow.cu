@@ -1363,6 +1363,7 @@ __global__ void k_chi_k(int nk, const double* __restrict__ kp, const T* __restri
 #include "tri.cuh"
 #include "tri_dense.cuh"
 #include "tri_adj.cuh"
+#include "pair_adj.cuh"
 
 // ----------------------------------------------------------------------------- objects
 
@@ -1439,6 +1440,11 @@ struct sr_flow {
     size_t smem_adj = 0;
     DevBuf<int> pinv_off, pinv_out, ainv_off, ainv_idx, binv_off, binv_idx;
     DevBuf<double> ntw, Wbar, dgbar, tg, tG, chibar, kbar;
+    bool pka_on = false;         // vertex adjoint on the packed state (pairk::k_gamma_adj_pair)
+    size_t pka_smem = 0;
+    DevBuf<int2> pka_list, pka_items;
+    DevBuf<int> pka_out_off, pka_out_idx;
+    DevBuf<double> Pbar;
     // TRI core tables (nc = 16)
     DevBuf<int> swap_map16, onsite_map16, tlat_item_off, tlat_off, chi_r16, chi_m16;
     DevBuf<int2> tlat_ent;
@@ -2489,6 +2495,61 @@ extern "C" sr_status sr_measure_susceptibility(sr_flow* f, int n_k, const double
 // gradient of a weighted sum of chi(k) with respect to the state.  The caller keeps (or
 // recomputes from checkpoints) the forward states and sets each with sr_flow_set_state.
 
+// The vertex adjoint on the packed state: inverted lattice-sum lists and accumulators.  Leaves
+// pka_on false (the general kernel serves the flow) where it does not fit.
+static sr_status adj_prepare_pair(sr_flow* f) {
+    const Geo& g = f->g;
+    if (!f->pk_on || f->prec != SR_FP64 || g.nc == 16) return SR_OK;
+    const int Ns = g.Ns, nc = g.nc, row = Ns * nc, np = f->nprod, nst = f->pk.nst;
+    const size_t sm = nc == 2 ? pairk::adj_smem<2>(g.N, Ns, f->pk.rv, nst, np) : pairk::adj_smem<4>(g.N, Ns, f->pk.rv, nst, np);
+    if (sm > 227 * 1024 || f->pk.rv / 2 > 128) return SR_OK;
+    // the fold needs the exchange to permute the stored entries
+    std::vector<int> hit(row, 0);
+    for (int r = 0; r < Ns; ++r)
+        for (int c = 0; c < nc; ++c)
+            if (hit[f->lat->swap_perm[r][c] * Ns + f->lat->swap_r[r]]++) return SR_OK;
+    std::vector<std::vector<int2>> lists(2 * row);
+    for (int i = 0; i < np; ++i) {
+        const int ra = f->h_prod[i].x / nc, ca = f->h_prod[i].x % nc, rb = f->h_prod[i].y / nc, cb = f->h_prod[i].y % nc;
+        lists[ca * Ns + ra].push_back(make_int2(i, cb * nst + rb));
+        lists[row + cb * Ns + rb].push_back(make_int2(i, ca * nst + ra));
+    }
+    size_t most = 1;
+    std::vector<int> off(np + 1, 0), idx(f->h_gidx.size());
+    std::vector<int2> items(2 * row);
+    for (int i = 0; i < 2 * row; ++i) { items[i] = make_int2(i, (int)lists[i].size()); most = std::max(most, lists[i].size()); }
+    std::stable_sort(items.begin(), items.end(), [](const int2& a, const int2& b) { return a.y > b.y; });
+    std::vector<int2> flat(most * 2 * row, make_int2(0, 0));
+    for (int i = 0; i < 2 * row; ++i)
+        for (int j = 0; j < items[i].y; ++j) flat[(size_t)j * 2 * row + i] = lists[items[i].x][j];
+    for (int u : f->h_gidx) off[u + 1]++;
+    for (int i = 0; i < np; ++i) off[i + 1] += off[i];
+    std::vector<int> fill(off.begin(), off.end() - 1);
+    for (int o = 0; o < row; ++o)   // h_goff runs over r * nc + c
+        for (int k = f->h_goff[o]; k < f->h_goff[o + 1]; ++k) idx[fill[f->h_gidx[k]]++] = (o % nc) * Ns + o / nc;
+    cudaStream_t st = f->stream;
+    if (f->Pbar.alloc(f->Pd.n) != cudaSuccess) {
+        cudaGetLastError();
+        f->Pbar.p = nullptr;
+        return SR_OK;
+    }
+    CK(f->pka_list.upload(flat.data(), flat.size(), st));
+    CK(f->pka_items.upload(items.data(), items.size(), st));
+    CK(f->pka_out_off.upload(off.data(), off.size(), st));
+    CK(f->pka_out_idx.upload(idx.data(), idx.size(), st));
+    CK(f->ntw.alloc((size_t)3 * g.N * g.nmax));
+    CK(f->Wbar.alloc((size_t)3 * g.N * g.nmax));
+    CK(f->dgbar.alloc((size_t)g.N));
+    CK(f->tg.alloc((size_t)g.N));
+    CK(f->tG.alloc((size_t)g.nent));
+    CK(ensure_smem(nc == 2 ? (const void*)pairk::k_gamma_adj_pair<2> : (const void*)pairk::k_gamma_adj_pair<4>, sm));
+    CK(cudaStreamSynchronize(st));
+    f->pka_smem = sm;
+    f->pka_on = true;
+    f->adj_ready = true;
+    return SR_OK;
+}
+
 static sr_status adj_prepare(sr_flow* f) {
     if (f->adj_ready) return SR_OK;
     const Geo& g = f->g;
@@ -2506,6 +2567,8 @@ static sr_status adj_prepare(sr_flow* f) {
         f->adj_ready = true;
         return SR_OK;
     }
+    if (sr_status s = adj_prepare_pair(f)) return s;
+    if (f->pka_on) return SR_OK;
     const int row = g.Ns * g.nc, np = f->nprod;
     std::vector<int> poff(np + 1, 0), pout(f->h_gidx.size());
     for (int o = 0; o < row; ++o)
@@ -2574,7 +2637,21 @@ static sr_status rhs_adjoint(sr_flow* f, double lam, const double* fbar_g, const
     if (g.nc == 16)
         k_gamma_adj_tri<<<blocks, kThreads, f->smem_adj, st>>>(g, tb, f->tabs_tri(), f->w.p, f->G.p, f->nx.p, f->nW.p,
                                                                f->ncount.p, fbar_G, Gbar_o, f->Wbar.p);
-    else if (g.nc == 2)
+    else if (f->pka_on) {
+        const pairk::AdjTab pa{f->pka_out_off.p, f->pka_out_idx.p, f->pka_list.p, f->pka_items.p};
+        const unsigned fb = (unsigned)std::min<long>((long)f->pk.nrow, 8192);
+        launch_pack_pair(f, f->G.p, st);
+        CK(cudaMemsetAsync(f->Pbar.p, 0, sizeof(double) * f->Pbar.n, st));
+        if (g.nc == 2) {
+            pairk::k_gamma_adj_pair<2><<<blocks, 128, f->pka_smem, st>>>(g, tb, f->pk, pa, f->Pd.p, f->nx.p, f->nW.p, f->ncount.p, fbar_G,
+                                                                         f->Pbar.p, f->Wbar.p);
+            pairk::k_pair_fold<2><<<fb, 64, sizeof(double) * g.Ns * 2, st>>>(g, tb, f->pk, f->Pbar.p, Gbar_o);
+        } else {
+            pairk::k_gamma_adj_pair<4><<<blocks, 128, f->pka_smem, st>>>(g, tb, f->pk, pa, f->Pd.p, f->nx.p, f->nW.p, f->ncount.p, fbar_G,
+                                                                         f->Pbar.p, f->Wbar.p);
+            pairk::k_pair_fold<4><<<fb, 64, sizeof(double) * g.Ns * 4, st>>>(g, tb, f->pk, f->Pbar.p, Gbar_o);
+        }
+    } else if (g.nc == 2)
         k_gamma_adj<2><<<blocks, kThreads, f->smem_adj, st>>>(g, tb, at, f->w.p, f->G.p, f->nx.p, f->nW.p, f->ncount.p,
                                                               fbar_G, Gbar_o, f->Wbar.p);
     else
