@@ -16,6 +16,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -117,30 +118,24 @@ __device__ void channel_nodes_block(Geo g, const double* __restrict__ w, const d
     const double inv2pi = 1.0 / (2.0 * kPi);
     const double wmax = w[N - 1];
     const int m = 2 * N + 4;
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < 4) {
         // delta points of the single-scale propagator, theta(0) = 1; a point whose partner
-        // propagator lies below the cutoff (theta = 0) contributes exactly zero
-        int n = 0;
-        for (int sg = 0; sg < 2; ++sg) {
-            double L = sg == 0 ? lam : -lam;
-            double a;
-            if (ch == 0) {          // G(w) S(s - w): w = s - L;  G(s - w) S(w): w = L
-                a = v - L;
-                const T vv = (fabs(a) - lam >= 0.0) ? T(prop_gg(w, invh, N, gam, a, L) * inv2pi) : T(0.0);
-                X[n] = a; Wt[n] = vv; ++n;
-                X[n] = L; Wt[n] = vv; ++n;
-            } else if (ch == 1) {   // G(w) S(w - t): w = t + L;  G(w - t) S(w): w = L
-                a = v + L;
-                X[n] = a; Wt[n] = (fabs(a) - lam >= 0.0) ? T(prop_gg(w, invh, N, gam, a, L) * inv2pi) : T(0.0); ++n;
-                a = L - v;
-                X[n] = L; Wt[n] = (fabs(a) - lam >= 0.0) ? T(prop_gg(w, invh, N, gam, a, L) * inv2pi) : T(0.0); ++n;
-            } else {                // G(w) S(u + w): w = L - u;  G(u + w) S(w): w = L
-                a = L - v;
-                X[n] = a; Wt[n] = (fabs(a) - lam >= 0.0) ? T(prop_gg(w, invh, N, gam, a, L) * inv2pi) : T(0.0); ++n;
-                a = v + L;
-                X[n] = L; Wt[n] = (fabs(a) - lam >= 0.0) ? T(prop_gg(w, invh, N, gam, a, L) * inv2pi) : T(0.0); ++n;
-            }
-        }
+        // propagator lies below the cutoff (theta = 0) contributes exactly zero:
+        //   s: G(w) S(s - w), w = s - L, and G(s - w) S(w), w = L (the same value)
+        //   t: G(w) S(w - t), w = t + L, and G(w - t) S(w), w = L
+        //   u: G(w) S(u + w), w = L - u, and G(u + w) S(w), w = L
+        const int n = threadIdx.x;
+        const double L = n < 2 ? lam : -lam;
+        double a;
+        if (ch == 0) a = v - L;
+        else if (ch == 1) a = (n & 1) ? L - v : v + L;
+        else a = (n & 1) ? v + L : L - v;
+        X[n] = (n & 1) ? L : a;
+        Wt[n] = (fabs(a) - lam >= 0.0) ? T(prop_gg(w, invh, N, gam, a, L) * inv2pi) : T(0.0);
+        if (Wf) Wf[n] = (float)value_of(Wt[n]);
+        if (nxf) nxf[(size_t)id * g.nmax + n] = (float)X[n];
+    }
+    if (threadIdx.x == blockDim.x - 1) {
         // break points, clipped to [-w_max, w_max], in ascending order (insertion order on ties)
         double q[4];
         if (ch == 2) { q[0] = lam; q[1] = -lam; q[2] = -v + lam; q[3] = -v - lam; }
@@ -186,21 +181,32 @@ __device__ void channel_nodes_block(Geo g, const double* __restrict__ w, const d
         twt[i] = wgt;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int n = 4;
-        for (int i = 0; i < m; ++i) {
-            if (!keep[i]) continue;
+    // compaction in order: ranks by warp ballots, a block's width of points at a time
+    __shared__ int wcount[32];
+    __shared__ int base_n;
+    if (threadIdx.x == 0) base_n = 4;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+    for (int i0 = 0; i0 < m; i0 += blockDim.x) {
+        const int i = i0 + threadIdx.x;
+        const bool k = i < m && keep[i];
+        const unsigned bal = __ballot_sync(0xffffffffu, k);
+        if (lane == 0) wcount[wid] = __popc(bal);
+        __syncthreads();
+        int n = base_n + __popc(bal & ((1u << lane) - 1u));
+        for (int q = 0; q < wid; ++q) n += wcount[q];
+        if (k) {
             X[n] = pts[i];
             Wt[n] = val[i];
             if (ntw) ntw[(size_t)id * g.nmax + n] = twt[i];
-            ++n;
+            if (Wf) Wf[n] = (float)value_of(val[i]);
+            if (nxf) nxf[(size_t)id * g.nmax + n] = (float)pts[i];
         }
-        if (Wf)
-            for (int i = 0; i < n; ++i) Wf[i] = (float)value_of(Wt[i]);
-        if (nxf)
-            for (int i = 0; i < n; ++i) nxf[(size_t)id * g.nmax + i] = (float)X[i];
-        ncount[id] = n;
+        __syncthreads();
+        if (threadIdx.x == 0)
+            for (int q = 0; q < nwarp; ++q) base_n += wcount[q];
+        __syncthreads();
     }
+    if (threadIdx.x == 0) ncount[id] = base_n;
 }
 
 template <typename T>
@@ -237,34 +243,44 @@ __device__ void block_sum(T (&v)[NV], double* red) {
 // Flow of the self-energy, one block per mesh frequency w_n:
 // dgamma(w) = -(1/2pi) sum_{w2 = +-Lambda} H(w, w2) / (w2 + gamma(w2)),
 // H = 2 sum_j Gamma^00_{ref j}(w+w2, 0, w-w2) - sum_c f_c Gamma^cc_{ref ref}(w+w2, w2-w, 0).
+// Four warps: Hartree and Fock part at w2 = +Lambda and -Lambda, so that their lookups overlap.
+constexpr int kSigmaThreads = 128;
+
 template <typename T>
 __device__ void sigma_rhs_block(Geo g, Tabs tb, const double* __restrict__ w, const T* __restrict__ gam,
                                 const T* __restrict__ G, double lam, T* __restrict__ dgam, const int n) {
-    __shared__ double red[2 * 32 * (sizeof(T) / sizeof(double))];
-    const double w1 = w[n];
-    T H[2] = {T(0.0), T(0.0)};
-    for (int sg = 0; sg < 2; ++sg) {
-        const double w2 = sg == 0 ? lam : -lam;
+    constexpr int D = sizeof(T) / sizeof(double);
+    __shared__ __align__(16) unsigned char part_raw[4 * sizeof(T)];
+    T* part = reinterpret_cast<T*>(part_raw);
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const double w1 = w[n], w2 = (wid & 1) ? -lam : lam;
+    if (wid < 4) {
         Desc<double> d;
-        make_desc(w1 + w2, 0.0, w1 - w2, 1, 0, tb, g, d);
         T h = T(0.0);
-        for (int r = threadIdx.x; r < g.Ns; r += blockDim.x) h += (double)tb.mult[r] * row_value(G, d, tb, g, r, 0);
-        h = 2.0 * h;
-        if (threadIdx.x == 0) {
-            Desc<double> e;
-            make_desc(w1 + w2, w2 - w1, 0.0, 2, 0, tb, g, e);
-            T f = T(0.0);
-            if (g.nc == 2) f = row_value(G, e, tb, g, 0, 0) + 3.0 * row_value(G, e, tb, g, 0, 1);
-            else for (int c = 0; c < 4; ++c) f += row_value(G, e, tb, g, 0, c);
-            h -= f;
+        if (wid < 2) {
+            make_desc(w1 + w2, 0.0, w1 - w2, 1, 0, tb, g, d);
+            for (int r = lane; r < g.Ns; r += 32) h += (double)tb.mult[r] * row_value(G, d, tb, g, r, 0);
+            h = 2.0 * h;
+        } else if (lane < g.nc) {
+            make_desc(w1 + w2, w2 - w1, 0.0, 2, 0, tb, g, d);
+            h = row_value(G, d, tb, g, 0, lane);
+            if (g.nc == 2 && lane == 1) h = 3.0 * h;
         }
-        H[sg] = h;
+        double* a = reinterpret_cast<double*>(&h);
+#pragma unroll
+        for (int k = 0; k < D; ++k)
+            for (int o = 16; o > 0; o >>= 1) a[k] += __shfl_down_sync(0xffffffffu, a[k], o);
+        if (lane == 0) part[wid] = h;
     }
-    block_sum<T, 2>(H, red);
+    __syncthreads();
+    if (wid < 2) {   // (both signs read gamma at once)
+        if (lane == 0) part[wid] = (part[wid] - part[2 + wid]) / (w2 + interp_odd(w, tb.invh, g.N, gam, w2));
+    }
+    __syncthreads();
     if (threadIdx.x == 0) {
         T acc = T(0.0);
-        acc += H[0] / (lam + interp_odd(w, tb.invh, g.N, gam, lam));
-        acc += H[1] / (-lam + interp_odd(w, tb.invh, g.N, gam, -lam));
+        acc += part[0];
+        acc += part[1];
         dgam[n] = -acc / (2.0 * kPi);
     }
 }
@@ -1215,12 +1231,15 @@ __global__ void k_fill_init(Geo g, const T* __restrict__ init /* Ns * nc */, T* 
 
 
 // y <- y + a f, flagging non-finite results.
-__global__ void k_axpy(long n, double* __restrict__ y, const double* __restrict__ f, double a, int* __restrict__ flag) {
+// Both parts of the state in one launch: gamma (n1 values), then Gamma (n2).
+__global__ void k_axpy(long n1, double* __restrict__ y1, const double* __restrict__ f1, long n2, double* __restrict__ y2,
+                       const double* __restrict__ f2, double a, int* __restrict__ flag) {
     long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    double v = y[i] + a * f[i];
+    if (i >= n1 + n2) return;
+    double* y = i < n1 ? y1 + i : y2 + (i - n1);
+    const double v = *y + a * (i < n1 ? f1[i] : f2[i - n1]);
     if (!isfinite(v)) atomicOr(flag, 1);
-    y[i] = v;
+    *y = v;
 }
 
 struct KPtrs { const double* k[7]; };
@@ -1358,6 +1377,7 @@ __global__ void k_chi_k(int nk, const double* __restrict__ kp, const T* __restri
 
 }  // namespace
 
+#include "chi.cuh"
 #include "adjoint.cuh"
 #include "pair.cuh"
 #include "tri.cuh"
@@ -1412,13 +1432,16 @@ struct sr_flow {
     size_t smem_tc = 0;           // dynamic shared memory of the tensor-core kernel
     int tc_grid = 0;              // its persistent grid (SMs x resident CTAs)
     int tc_occ_api = 0;           // the runtime's occupancy figure for it (reported only)
-    DevBuf<int> tcfail;           // set by the tensor-core kernel when an MMA wait gives up
     int nprod = 0;
     DevBuf<double> init;
     DevBuf<int2> chi_map;
     DevBuf<int> chi_onsite;
     DevBuf<double> chi_dr, chi, kbuf, chik;
-    DevBuf<int> flag;
+    // correlations of the SU2 / XYZ cores (chik::): displacements merged up to sign, partial sums
+    DevBuf<double> chi_d, chi_sd, chi_part;
+    DevBuf<int> chi_doff, chi_dpair, chi_counter;
+    int chi_nd = 0;
+    DevBuf<int> flag;             // [0] non-finite value, [1] the tensor-core kernel's MMA wait gave up
     DevBuf<unsigned long long> errbits;
     // Dormand-Prince work space (allocated on first use)
     DevBuf<double> y0g, y0G, stg, stG;
@@ -1533,13 +1556,15 @@ static sr_status prof_end(sr_flow* f, int id, cudaEvent_t b) {
 static void launch_pack_pair(sr_flow* f, const double* G_s, cudaStream_t st) {
     const Geo& g = f->g;
     const Tabs tb = f->tabs();
-    const unsigned nb = (unsigned)std::min<long>(((long)f->pk.nrow * g.Ns + 255) / 256, 8192);
+    const int RB = std::max(1, pairk::kPackThreads / g.Ns);
+    const unsigned nb = (unsigned)std::min<long>(((long)f->pk.nrow + RB - 1) / RB, 8192);
+    constexpr int th = pairk::kPackThreads;
     if (f->prec == SR_FP64) {
-        if (g.nc == 2) pairk::k_pair_pack<double, 2><<<nb, 256, 0, st>>>(g, tb, f->pk, G_s, f->Pd.p);
-        else pairk::k_pair_pack<double, 4><<<nb, 256, 0, st>>>(g, tb, f->pk, G_s, f->Pd.p);
+        if (g.nc == 2) pairk::k_pair_pack<double, 2><<<nb, th, pairk::pack_smem<double, 2>(g.Ns), st>>>(g, tb, f->pk, G_s, f->Pd.p);
+        else pairk::k_pair_pack<double, 4><<<nb, th, pairk::pack_smem<double, 4>(g.Ns), st>>>(g, tb, f->pk, G_s, f->Pd.p);
     } else {
-        if (g.nc == 2) pairk::k_pair_pack<float, 2><<<nb, 256, 0, st>>>(g, tb, f->pk, G_s, f->Pf.p);
-        else pairk::k_pair_pack<float, 4><<<nb, 256, 0, st>>>(g, tb, f->pk, G_s, f->Pf.p);
+        if (g.nc == 2) pairk::k_pair_pack<float, 2><<<nb, th, pairk::pack_smem<float, 2>(g.Ns), st>>>(g, tb, f->pk, G_s, f->Pf.p);
+        else pairk::k_pair_pack<float, 4><<<nb, th, pairk::pack_smem<float, 4>(g.Ns), st>>>(g, tb, f->pk, G_s, f->Pf.p);
     }
 }
 
@@ -1612,7 +1637,7 @@ static sr_status run_rhs(sr_flow* f, double lam, const double* gam_s, const doub
         if (g.nc == 16)
             k_sigma_rhs_tri<DualT><<<g.N, 64, 0, f->stream>>>(g, tb, f->tabs_tri(), f->w.p, gs, Gd, lam, dgo);
         else
-            k_sigma_rhs<DualT><<<g.N, 64, 0, f->stream>>>(g, tb, f->w.p, gs, Gd, lam, dgo);
+            k_sigma_rhs<DualT><<<g.N, kSigmaThreads, 0, f->stream>>>(g, tb, f->w.p, gs, Gd, lam, dgo);
         if (sr_status s = prof_end(f, 0, e0)) return s;
         if (sr_status s = prof_begin(f, 1, &e0)) return s;
         k_channel_nodes<DualT><<<3 * g.N, 128, 0, f->stream>>>(g, f->w.p, f->invh.p, gs, dgo, lam, f->nx.p, nW, nullptr, f->ncount.p,
@@ -1649,7 +1674,7 @@ static sr_status run_rhs(sr_flow* f, double lam, const double* gam_s, const doub
         return SR_OK;
     }
     if (sr_status s = prof_begin(f, 0, &e0)) return s;
-    k_sigma_rhs<double><<<g.N, 64, 0, f->stream>>>(g, tb, f->w.p, gam_s, G_s, lam, dgam_o);
+    k_sigma_rhs<double><<<g.N, kSigmaThreads, 0, f->stream>>>(g, tb, f->w.p, gam_s, G_s, lam, dgam_o);
     if (sr_status s = prof_end(f, 0, e0)) return s;
     if (sr_status s = prof_begin(f, 1, &e0)) return s;
     k_channel_nodes<double><<<3 * g.N, 128, 0, f->stream>>>(g, f->w.p, f->invh.p, gam_s, dgam_o, lam, f->nx.p, f->nW.p, f->nWf.p,
@@ -1670,7 +1695,7 @@ static sr_status run_rhs(sr_flow* f, double lam, const double* gam_s, const doub
             k_shadow<<<(unsigned)((g.nentp + 255) / 256), 256, 0, f->stream>>>(g, tb, G_s, f->Gf.p, f->has_swap ? 1 : 0);
         if (g.nc == 2 && f->dense && f->use_tc)
             k_gamma_rhs_f32_tc<<<std::min(blocks, f->tc_grid), kThreads, f->smem_tc, f->stream>>>(g, tb, Gf_s, Gs, f->nxf.p, f->nWf.p, f->ncount.p, dG_o,
-                                                                            f->tcfail.p, (long)pb * g.N, (long)pe * g.N);
+                                                                            f->flag.p + 1, (long)pb * g.N, (long)pe * g.N);
         else if (g.nc == 2 && f->dense)
             k_gamma_rhs_f32<2, true><<<blocks, kThreads, f->smem_rhs, f->stream>>>(g, tb, Gf_s, Gs, f->nxf.p, f->nWf.p, f->ncount.p, dG_o, pb);
         else if (g.nc == 2)
@@ -1942,6 +1967,19 @@ static sr_status flow_create(const sr_lattice* lat, int n_freq, const double* fr
         CK(f->chi_onsite.upload(lat->chi_onsite.data(), lat->chi_onsite.size(), st));
         CK(f->chi_dr.upload(lat->chi_dr.data(), lat->chi_dr.size(), st));
         CK(f->chi.alloc(lat->chi_map.size() * g.nc * ts));
+        if (g.nc != 16 && !f->ntan) {
+            const chik::Displacements D = chik::merge(lat->chi_dr);
+            f->chi_nd = (int)D.off.size() - 1;
+            CK(f->chi_d.upload(D.dr.data(), D.dr.size(), st));
+            CK(f->chi_doff.upload(D.off.data(), D.off.size(), st));
+            CK(f->chi_dpair.upload(D.pair.data(), D.pair.size(), st));
+            CK(f->chi_sd.alloc(f->chi_nd));
+            CK(f->chi_part.alloc(chik::part_doubles(g.Ns, g.nc)));
+            CK(f->chi_counter.alloc(1));
+            CK(cudaMemsetAsync(f->chi_counter.p, 0, sizeof(int), st));
+            const size_t sm = sizeof(double) * 2 * g.Ns * g.nc * chik::groups(g.Ns * g.nc);
+            if (sm > 32 * 1024) CK(ensure_smem(g.nc == 2 ? (const void*)chik::k_chi_sum<2> : (const void*)chik::k_chi_sum<4>, sm));
+        }
     }
     if (lat->nc == 16) {
         // TRI core: component maps and the lattice-sum table: per entry (rA, mA, rB, mB) of an
@@ -2080,7 +2118,8 @@ static sr_status flow_create(const sr_lattice* lat, int n_freq, const double* fr
     CK(f->nWf.alloc((size_t)3 * g.N * g.nmax));
     CK(f->nxf.alloc((size_t)3 * g.N * g.nmax));
     CK(f->ncount.alloc((size_t)3 * g.N));
-    CK(f->flag.alloc(1));
+    CK(f->flag.alloc(2));
+    CK(cudaMemsetAsync(f->flag.p, 0, 2 * sizeof(int), st));
     CK(f->errbits.alloc(2));
     CK(cudaMemsetAsync(f->gam.p, 0, sizeof(double) * g.N * ts, st));
     if (f->ntan)
@@ -2098,8 +2137,6 @@ static sr_status flow_create(const sr_lattice* lat, int n_freq, const double* fr
     if (tc_ok) f->smem_tc = f32_smem_bytes(g.Ns, g.nsp, g.nc, f->nprod, f->dense, true);
     f->use_tc = false;   // off by default: slower than the CUDA-core contraction on the square
                          // J1-J2 and pyrochlore workloads (operand staging outweighs the contraction)
-    CK(f->tcfail.alloc(1));
-    CK(cudaMemsetAsync(f->tcfail.p, 0, sizeof(int), st));
     if (f->smem_rhs > 227 * 1024) return fail(SR_EUNSUPPORTED, "lattice too large for one CTA's shared memory (%zu bytes)", f->smem_rhs);
     if (g.nc == 16) {
         if (f->ntan) CK(ensure_smem((const void*)k_gamma_rhs_tri<DualT>, f->smem_rhs));
@@ -2197,10 +2234,10 @@ extern "C" sr_status sr_flow_rhs(sr_flow* f, double lambda, double* d_dsigma, do
 }
 
 static sr_status check_flag(sr_flow* f, double lam) {
-    int h = 0, t = 0;
-    CK(cudaMemcpyAsync(&h, f->flag.p, sizeof(int), cudaMemcpyDeviceToHost, f->stream));
-    CK(cudaMemcpyAsync(&t, f->tcfail.p, sizeof(int), cudaMemcpyDeviceToHost, f->stream));
+    int ht[2] = {0, 0};
+    CK(cudaMemcpyAsync(ht, f->flag.p, 2 * sizeof(int), cudaMemcpyDeviceToHost, f->stream));
     CK(cudaStreamSynchronize(f->stream));
+    const int h = ht[0], t = ht[1];
     if (t) return fail(SR_ETIMEOUT, "tensor-core MMA completion wait gave up (Lambda = %.17g)", lam);
     if (h) return fail(SR_ENONFINITE, "non-finite value in the flow at Lambda = %.17g", lam);
     return SR_OK;
@@ -2212,8 +2249,8 @@ static sr_status euler_step(sr_flow* f, double lam_next) {
     if (sr_status s = run_rhs(f, f->lambda, f->gam.p, f->G.p, f->Gf.p, f->dgam.p, f->dG.p)) return s;
     CK(cudaMemsetAsync(f->flag.p, 0, sizeof(int), f->stream));
     const long nG = g.nent * f->ts;
-    k_axpy<<<1, 256, 0, f->stream>>>((long)g.N * f->ts, f->gam.p, f->dgam.p, -dl, f->flag.p);
-    k_axpy<<<(unsigned)((nG + 255) / 256), 256, 0, f->stream>>>(nG, f->G.p, f->dG.p, -dl, f->flag.p);
+    const long n1 = (long)g.N * f->ts;
+    k_axpy<<<(unsigned)((n1 + nG + 255) / 256), 256, 0, f->stream>>>(n1, f->gam.p, f->dgam.p, nG, f->G.p, f->dG.p, -dl, f->flag.p);
     CK(cudaGetLastError());
     if (sr_status s = refresh_shadow(f, f->G.p, f->Gf.p)) return s;
     if (sr_status s = check_flag(f, lam_next)) return s;
@@ -2243,8 +2280,8 @@ extern "C" sr_status sr_flow_advance(sr_flow* f, double lambda_next, const doubl
     const double dl = f->lambda - lambda_next;
     CK(cudaMemsetAsync(f->flag.p, 0, sizeof(int), f->stream));
     const long nG = g.nent * f->ts;
-    k_axpy<<<1, 256, 0, f->stream>>>((long)g.N * f->ts, f->gam.p, d_dsigma, -dl, f->flag.p);
-    k_axpy<<<(unsigned)((nG + 255) / 256), 256, 0, f->stream>>>(nG, f->G.p, d_dgamma, -dl, f->flag.p);
+    const long n1 = (long)g.N * f->ts;
+    k_axpy<<<(unsigned)((n1 + nG + 255) / 256), 256, 0, f->stream>>>(n1, f->gam.p, d_dsigma, nG, f->G.p, d_dgamma, -dl, f->flag.p);
     CK(cudaGetLastError());
     if (sr_status s = refresh_shadow(f, f->G.p, f->Gf.p)) return s;
     if (sr_status s = check_flag(f, lambda_next)) return s;
@@ -2456,6 +2493,26 @@ extern "C" sr_status sr_measure_susceptibility_tangent(sr_flow* f, int n_k, cons
     return SR_OK;
 }
 
+// chi_ij of an SU2 / XYZ flow into chi (and the displacement sums that chi(k) reads).  Blocks take at
+// least 16 frequency pairs each.
+static void launch_chi(sr_flow* f, double* chi) {
+    const Geo& g = f->g;
+    const Tabs tb = f->tabs();
+    const int npairs = (int)f->lat->chi_map.size();
+    int K = 1;
+    for (double w : f->mesh) K += w > f->lambda;
+    const int nb = std::max(1, std::min(chik::kMaxBlocks, (2 * K * K + 15) / 16));
+    const size_t sm = sizeof(double) * 2 * g.Ns * g.nc * chik::groups(g.Ns * g.nc);
+    if (g.nc == 2)
+        chik::k_chi_sum<2><<<nb, chik::kThreads, sm, f->stream>>>(g, tb, f->w.p, f->gam.p, f->G.p, f->lambda, f->chi_map.p, f->chi_onsite.p,
+                                                                  f->lat->Ntot, npairs, f->chi_doff.p, f->chi_dpair.p, f->chi_nd,
+                                                                  f->chi_part.p, f->chi_counter.p, chi, f->chi_sd.p);
+    else
+        chik::k_chi_sum<4><<<nb, chik::kThreads, sm, f->stream>>>(g, tb, f->w.p, f->gam.p, f->G.p, f->lambda, f->chi_map.p, f->chi_onsite.p,
+                                                                  f->lat->Ntot, npairs, f->chi_doff.p, f->chi_dpair.p, f->chi_nd,
+                                                                  f->chi_part.p, f->chi_counter.p, chi, f->chi_sd.p);
+}
+
 extern "C" sr_status sr_measure_susceptibility(sr_flow* f, int n_k, const double* k_xyz, double* chi_k, double* chi_ij) {
     if (!f) return fail(SR_EINVAL, "null flow");
     if (f->ntan) return fail(SR_EINVAL, "tangent flows measure with sr_measure_susceptibility_tangent");
@@ -2467,10 +2524,8 @@ extern "C" sr_status sr_measure_susceptibility(sr_flow* f, int n_k, const double
     if (g.nc == 16)
         k_chi_tri<<<npairs, 128, 0, f->stream>>>(g, tb, f->tabs_tri(), f->w.p, f->gam.p, f->G.p, f->lambda, f->chi_r16.p, f->chi_m16.p,
                                                  f->chi_onsite.p, lat->Ntot, f->chi.p);
-    else if (g.nc == 2)
-        k_chi<double, 2><<<npairs, 128, 0, f->stream>>>(g, tb, f->w.p, f->gam.p, f->G.p, f->lambda, f->chi_map.p, f->chi_onsite.p, lat->Ntot, f->chi.p);
     else
-        k_chi<double, 4><<<npairs, 128, 0, f->stream>>>(g, tb, f->w.p, f->gam.p, f->G.p, f->lambda, f->chi_map.p, f->chi_onsite.p, lat->Ntot, f->chi.p);
+        launch_chi(f, f->chi.p);
     CK(cudaGetLastError());
     if (chi_ij) CK(cudaMemcpyAsync(chi_ij, f->chi.p, sizeof(double) * npairs * g.nc, cudaMemcpyDeviceToDevice, f->stream));
     if (chi_k && n_k > 0) {
@@ -2480,7 +2535,7 @@ extern "C" sr_status sr_measure_susceptibility(sr_flow* f, int n_k, const double
         if (g.nc == 16)
             k_chi_k_tri<<<(n_k + 127) / 128, 128, 0, f->stream>>>(n_k, f->kbuf.p, f->chi.p, f->chi_dr.p, npairs, lat->nb, f->chik.p);
         else
-            k_chi_k<double><<<(n_k + 127) / 128, 128, 0, f->stream>>>(n_k, f->kbuf.p, f->chi.p, f->chi_dr.p, npairs, lat->nb, g.nc, f->chik.p);
+            chik::k_chi_fourier<<<(n_k + 3) / 4, chik::kThreads, 0, f->stream>>>(n_k, f->kbuf.p, f->chi_d.p, f->chi_sd.p, f->chi_nd, lat->nb, f->chik.p);
         CK(cudaGetLastError());
         CK(cudaMemcpyAsync(chi_k, f->chik.p, sizeof(double) * n_k, cudaMemcpyDeviceToHost, f->stream));
         CK(cudaStreamSynchronize(f->stream));
@@ -2626,7 +2681,7 @@ static sr_status rhs_adjoint(sr_flow* f, double lam, const double* fbar_g, const
     if (g.nc == 16)
         k_sigma_rhs_tri<double><<<g.N, 64, 0, st>>>(g, tb, f->tabs_tri(), f->w.p, f->gam.p, f->G.p, lam, f->dgam.p);
     else
-        k_sigma_rhs<double><<<g.N, 64, 0, st>>>(g, tb, f->w.p, f->gam.p, f->G.p, lam, f->dgam.p);
+        k_sigma_rhs<double><<<g.N, kSigmaThreads, 0, st>>>(g, tb, f->w.p, f->gam.p, f->G.p, lam, f->dgam.p);
     k_channel_nodes<double><<<3 * g.N, 128, 0, st>>>(g, f->w.p, f->invh.p, f->gam.p, f->dgam.p, lam, f->nx.p, f->nW.p,
                                                      nullptr, f->ncount.p, nullptr, f->ntw.p);
     CK(cudaMemsetAsync(gbar_o, 0, sizeof(double) * g.N, st));
@@ -2994,11 +3049,9 @@ __global__ void k_pack_b(const BInst* __restrict__ I) {
     const Geo g = B.g;
     const Tabs tb = B.tb;
     const pairk::Tab td = B.pk;
-    const long n = (long)td.nrow * g.Ns;
-    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-        if (g.nc == 2) pairk::pack_site<float, 2>(g, tb, td, B.G, B.P, i);
-        else pairk::pack_site<float, 4>(g, tb, td, B.G, B.P, i);
-    }
+    extern __shared__ __align__(16) unsigned char smem[];
+    if (g.nc == 2) pairk::pack_rows<float, 2>(g, tb, td, B.G, B.P, smem);
+    else pairk::pack_rows<float, 4>(g, tb, td, B.G, B.P, smem);
 }
 
 __global__ void k_advance(int* __restrict__ step, unsigned long long* __restrict__ counter, int ncounter) {
@@ -3097,10 +3150,16 @@ static sr_status launch_classes(sr_batch* b) {
 
 static void batch_pack(sr_batch* b) {
     long most = 0;
+    size_t sm = 0;
     for (const BInst& B : b->inst)
-        if (B.kind == 0) most = std::max(most, (long)B.pk.nrow * B.g.Ns);
+        if (B.kind == 0) {
+            const int RB = std::max(1, pairk::kPackThreads / B.g.Ns);
+            most = std::max(most, ((long)B.pk.nrow + RB - 1) / RB);
+            sm = std::max(sm, pairk::pack_smem<float, 4>(B.g.Ns));
+        }
     if (most > 0)
-        k_pack_b<<<dim3((unsigned)std::min<long>((most + 255) / 256, 4 * b->nsm), (unsigned)b->inst.size()), 256, 0, b->stream>>>(b->dinst.p);
+        k_pack_b<<<dim3((unsigned)std::min<long>(most, 8 * b->nsm), (unsigned)b->inst.size()), pairk::kPackThreads, sm, b->stream>>>(
+            b->dinst.p);
 }
 
 static sr_status batch_launch_step(sr_batch* b) {
@@ -3108,7 +3167,7 @@ static sr_status batch_launch_step(sr_batch* b) {
     int maxN = 0;
     long maxent = 0;
     for (const BInst& B : b->inst) { maxN = std::max(maxN, B.g.N); maxent = std::max(maxent, B.g.nentp); }
-    k_sigma_b<<<dim3(maxN, ni), 64, 0, b->stream>>>(b->dinst.p, b->lams.p, b->step.p);
+    k_sigma_b<<<dim3(maxN, ni), kSigmaThreads, 0, b->stream>>>(b->dinst.p, b->lams.p, b->step.p);
     k_nodes_b<<<dim3(3 * maxN, ni), 128, 0, b->stream>>>(b->dinst.p, b->lams.p, b->step.p);
     batch_pack(b);
     if (sr_status s = launch_classes(b)) return s;
@@ -3396,7 +3455,7 @@ extern "C" sr_status sr_batch_run(sr_batch* b, int n_lambda, const double* lambd
         for (const BInst& B : b->inst) maxN = std::max(maxN, B.g.N);
         const int mid = nsteps / 2;
         CK(cudaMemcpyAsync(b->step.p, &mid, sizeof(int), cudaMemcpyHostToDevice, b->stream));
-        k_sigma_b<<<dim3(maxN, ni), 64, 0, b->stream>>>(b->dinst.p, b->lams.p, b->step.p);
+        k_sigma_b<<<dim3(maxN, ni), kSigmaThreads, 0, b->stream>>>(b->dinst.p, b->lams.p, b->step.p);
         k_nodes_b<<<dim3(3 * maxN, ni), 128, 0, b->stream>>>(b->dinst.p, b->lams.p, b->step.p);
         batch_pack(b);
         CK(cudaGetLastError());
@@ -3534,16 +3593,14 @@ extern "C" sr_status sr_measure_susceptibility_static(sr_flow* f, int n_k, const
     if (g.nc == 16)
         k_chi_tri<<<npairs, 128, 0, f->stream>>>(g, tb, f->tabs_tri(), f->w.p, f->gam.p, f->G.p, f->lambda, f->chi_r16.p, f->chi_m16.p,
                                                  f->chi_onsite.p, lat->Ntot, scratch);
-    else if (g.nc == 2)
-        k_chi<double, 2><<<npairs, 128, 0, f->stream>>>(g, tb, f->w.p, f->gam.p, f->G.p, f->lambda, f->chi_map.p, f->chi_onsite.p, lat->Ntot, scratch);
     else
-        k_chi<double, 4><<<npairs, 128, 0, f->stream>>>(g, tb, f->w.p, f->gam.p, f->G.p, f->lambda, f->chi_map.p, f->chi_onsite.p, lat->Ntot, scratch);
+        launch_chi(f, scratch);
     CK(cudaGetLastError());
     if (n_k > 0) {
         if (g.nc == 16)
             k_chi_k_tri<<<(n_k + 127) / 128, 128, 0, f->stream>>>(n_k, d_k_xyz, scratch, f->chi_dr.p, npairs, lat->nb, d_chi_k);
         else
-            k_chi_k<double><<<(n_k + 127) / 128, 128, 0, f->stream>>>(n_k, d_k_xyz, scratch, f->chi_dr.p, npairs, lat->nb, g.nc, d_chi_k);
+            chik::k_chi_fourier<<<(n_k + 3) / 4, chik::kThreads, 0, f->stream>>>(n_k, d_k_xyz, f->chi_d.p, f->chi_sd.p, f->chi_nd, lat->nb, d_chi_k);
         CK(cudaGetLastError());
     }
     return SR_OK;

@@ -515,42 +515,100 @@ k_gamma_rhs_pair(Geo g, Tabs tb, Tab td, const R* __restrict__ P, const R* __res
     triple<R, NC, TM, TN, NT>(g, tb, td, P, nx, nW, ncount, dG, p0 + (int)(blockIdx.x / g.N), blockIdx.x % g.N, smem);
 }
 
-// Packed state: s and u eigenvalue rows and component rows of every stored triple, and the same of
-// the exchanged pairs when the site exchange is not trivial (the padding stays zero).
-template <typename R, int NC>
-__device__ __forceinline__ void pack_site(const Geo& g, const Tabs& tb, const Tab& td, const double* __restrict__ G,
-                                          R* __restrict__ P, long i) {
-    const long row = i / g.Ns;
-    const int r = (int)(i - row * g.Ns);
-    const double* src = G + (size_t)row * NC * g.Ns;
-    for (int x = 0; x < (td.ex_t ? 2 : 1); ++x) {
-        const int rs = x ? tb.swap_r[r] : r, pm = x ? tb.swap_perm[r] : 0xe4;
-        double v[NC];
+// Eigenvalue e of components given as float pairs (hi + lo), rounded once: the sum of the FP64
+// components in FP32 arithmetic (two-term sums with their exact error, Knuth 1969).  FP64 additions and
+// conversions would bound the packing (36 per site for XYZ, 2 per clock and SM).
+template <int NC>
+__device__ __forceinline__ float eigen_pair(const float* hi, const float* lo, int e, int SGN) {
+    float h = hi[0], l = lo[0];
+    auto add = [&](float x, float xl) {
+        const float t = h + x, b = t - h;
+        l += (h - (t - b)) + (x - b) + xl;
+        h = t;
+    };
+    if (NC == 2) {
+        const bool pos = (SGN > 0) == (e == 0);
+        const float x = pos ? hi[1] : -hi[1], xl = pos ? lo[1] : -lo[1];
+        add(x, xl);
+        if (e == 1) add(2.0f * x, 2.0f * xl);
+    } else {
 #pragma unroll
-        for (int c = 0; c < NC; ++c) v[c] = src[perm_of(pm, c) * g.Ns + rs];
-        R* ps = P + (size_t)(x ? td.ex_su : 0) + (size_t)row * td.rv + r;
-        R* pt = P + td.su_t + (size_t)(x ? td.ex_t : 0) + (size_t)row * NC * td.nst + r;
-#pragma unroll
-        for (int c = 0; c < NC; ++c) {
-            ps[c * g.Ns] = (R)eigen<NC, double>(v, c, 1);
-            ps[td.su_u + c * g.Ns] = (R)eigen<NC, double>(v, c, -1);
-            pt[c * td.nst] = (R)v[c];
-            if (x == 0 && r == 0) {
-                R* on = P + td.on + (size_t)row * 2 * NC + c;
-                const int ti = (int)(row % g.N);
-                on[0] = (R)v[c];
-                if (ti > 0) on[-NC] = (R)v[c];
-                if (ti == g.N - 1) on[NC] = (R)v[c];
-            }
+        for (int c = 1; c < NC; ++c) {
+            const bool pos = SGN * bell(e, c) > 0;
+            add(pos ? hi[c] : -hi[c], pos ? lo[c] : -lo[c]);
         }
+    }
+    return h + l;
+}
+
+// Packed state: s and u eigenvalue rows and component rows of every stored triple, and the same of
+// the exchanged pairs when the site exchange is not trivial (the padding stays zero).  A block takes
+// whole rows, staged in shared memory (FP32: as float pairs), so that a component is read and
+// converted once; kPackThreads threads, grid-stride over the rows.
+constexpr int kPackThreads = 256;
+template <typename R, int NC> __host__ __device__ constexpr size_t pack_smem(int Ns) {
+    return sizeof(double) * NC * (kPackThreads > Ns ? kPackThreads : Ns);
+}
+
+template <typename R, int NC>
+__device__ __forceinline__ void pack_rows(const Geo& g, const Tabs& tb, const Tab& td, const double* __restrict__ G,
+                                          R* __restrict__ P, unsigned char* smem) {
+    const int Ns = g.Ns, RB = max(1, kPackThreads / Ns), cap = RB * Ns;   // rows of a block, their sites
+    R* sh = reinterpret_cast<R*>(smem);                                   // [component][site] (and the low parts)
+    const bool small = Ns <= kPackThreads;
+    const int my_row = small ? (int)threadIdx.x / Ns : 0, first = small ? (int)threadIdx.x - my_row * Ns : (int)threadIdx.x;
+    for (int row0 = blockIdx.x * RB; row0 < td.nrow; row0 += gridDim.x * RB) {
+        const int row = row0 + my_row;
+        const bool on = my_row < RB && row < td.nrow;
+        const double* src = G + (size_t)row * NC * Ns;
+        for (int r = first; on && r < Ns; r += kPackThreads)
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                const double x = src[c * Ns + r];
+                const R h = (R)x;
+                sh[c * cap + my_row * Ns + r] = h;
+                if (sizeof(R) == 4) sh[(NC + c) * cap + my_row * Ns + r] = isfinite(h) ? (R)(x - (double)h) : R(0);
+            }
+        __syncthreads();
+        for (int r = first; on && r < Ns; r += kPackThreads)
+            for (int x = 0; x < (td.ex_t ? 2 : 1); ++x) {
+                const int rs = my_row * Ns + (x ? tb.swap_r[r] : r), pm = x ? tb.swap_perm[r] : 0xe4;
+                R v[NC], lo[NC];
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    const int cs = perm_of(pm, c);
+                    v[c] = sh[cs * cap + rs];
+                    lo[c] = sizeof(R) == 4 ? sh[(NC + cs) * cap + rs] : R(0);
+                }
+                R* ps = P + (size_t)(x ? td.ex_su : 0) + (size_t)row * td.rv + r;
+                R* pt = P + td.su_t + (size_t)(x ? td.ex_t : 0) + (size_t)row * NC * td.nst + r;
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    if constexpr (sizeof(R) == 4) {
+                        ps[c * Ns] = eigen_pair<NC>(v, lo, c, 1);
+                        ps[td.su_u + c * Ns] = eigen_pair<NC>(v, lo, c, -1);
+                    } else {
+                        ps[c * Ns] = eigen<NC, R>(v, c, 1);
+                        ps[td.su_u + c * Ns] = eigen<NC, R>(v, c, -1);
+                    }
+                    pt[c * td.nst] = v[c];
+                    if (x == 0 && r == 0) {
+                        R* o = P + td.on + (size_t)row * 2 * NC + c;
+                        const int ti = row % g.N;
+                        o[0] = v[c];
+                        if (ti > 0) o[-NC] = v[c];
+                        if (ti == g.N - 1) o[NC] = v[c];
+                    }
+                }
+            }
+        __syncthreads();
     }
 }
 
 template <typename R, int NC>
-__global__ void k_pair_pack(Geo g, Tabs tb, Tab td, const double* __restrict__ G, R* __restrict__ P) {
-    const long n = (long)td.nrow * g.Ns;
-    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
-        pack_site<R, NC>(g, tb, td, G, P, i);
+__global__ void __launch_bounds__(kPackThreads) k_pair_pack(Geo g, Tabs tb, Tab td, const double* __restrict__ G, R* __restrict__ P) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    pack_rows<R, NC>(g, tb, td, G, P, smem);
 }
 
 // ---- host side
