@@ -167,47 +167,53 @@ def _job_throughput(units_per_rank: float, ws: int, t_ms: float) -> float:
     return units_per_rank * ws / (t_ms * 1e-3)
 
 
-def _algorithmic_flops(counts: np.ndarray, N: int, Ns: int, nc: int, P: int, nprod: int) -> float:
-    """Floating-point operations of one vertex-flow launch, counted as the natural evaluation
-    of the flow equations (an FMA = 2 flop).  Per stored triple (s, t, u) and integration node:
-    every vertex row the equations need is interpolated over all irreducible sites and
-    components; one of the three frequency arguments of every row is a mesh frequency, so an
-    interpolated value is 4 corners = 4 FMA = 8 flop, and the node weight multiplies one row
-    (1 flop per value).  s and u channels: two rows and the projected product (SU2 11 flop per
-    site: A1 B1, its multiples and three FMAs plus two accumulations; XYZ 32).  t channel: two
-    rows, two on-site rows (n_c values each), the on-site terms (SU2 6 flop per site and
-    component, XYZ 7) and the lattice sum as one FMA (2 flop) per distinct product of table
-    rows.  Per triple, the lattice sum's table gather adds P n_c flop.  TRI (n_c = 16): the
-    s / u products are 256 FMA per site (512 flop), the two on-site terms 1024 flop per site
-    (64 per value), and the lattice sum 64 FMA per table entry (nprod = 64 P), summed in
-    place."""
-    row = Ns * nc
-    prod = {2: 11, 4: 32, 16: 512}[nc]
-    onsite = {2: 6, 4: 7, 16: 64}[nc]
-    per_s = 2 * row * 8 + row + Ns * prod
+def _graded(model) -> bool:
+    """Whether some spin axis a has J^{ab} = J^{ba} = 0 for b != a on every coupling: only 8 of the
+    16 TRI functions are then non-zero (their spin indices both in {0, a} or both outside)."""
+    return any(all(abs(c.M[a, b]) < 1e-12 and abs(c.M[b, a]) < 1e-12 for c in model.couplings for b in range(3) if b != a)
+               for a in range(3))
+
+
+def _algorithmic_flops(counts: np.ndarray, N: int, Ns: int, nc: int, P: int, nprod: int, graded: bool = False) -> float:
+    """Floating-point operations of one vertex-flow launch, as the vertex kernels evaluate the flow
+    equations (an FMA = 2 flop).  Per stored triple (s, t, u) and integration node: every vertex row
+    the equations need is interpolated over all irreducible sites and components; one of the three
+    frequency arguments of every row is a mesh frequency, so an interpolated value is 4 corners =
+    4 FMA = 8 flop (node weights ride on corner weights).  s and u channels: two rows and one FMA per
+    value (products of eigenvalues).  t channel: two rows, two on-site rows (n_c values each), the
+    on-site terms (two FMA per value) and the lattice sum as one FMA per distinct product of table
+    rows.  TRI (n_c = 16, or 8 with a graded vertex): s / u products n_c x 16 (8) FMA per site, the two
+    on-site terms 4 (2) FMA each per value, the lattice sum 64 (16) FMA per pair of sites at most."""
+    if nc == 16:
+        m = 8 if graded else 16
+        row = Ns * m
+        prod, onsite = 2 * m * m * Ns, (8 if graded else 16) * row
+        lat_flop = 2 * (16 if graded else 64) * min(P, Ns * Ns)
+    else:
+        m, row = nc, Ns * nc
+        prod, onsite, lat_flop = 2 * row, 4 * row, 2 * nprod
+    per_s = 2 * row * 8 + prod
     per_u = per_s
-    per_t = (2 * row + 2 * nc) * 8 + row + nc + 2 * nprod + onsite * row
+    per_t = (2 * row + 2 * m) * 8 + lat_flop + onsite
     ns, nt, nu = counts[0].astype(np.float64), counts[1].astype(np.float64), counts[2].astype(np.float64)
     cs = np.arange(1, N + 1, dtype=np.float64)   # number of u_i <= s_i
     tot = N * float(np.sum(ns * cs)) * per_s                   # s channel: node count depends on s_i
     tot += (N * (N + 1) / 2) * float(np.sum(nt)) * per_t       # t channel: on t_i
     tot += N * float(np.sum(nu * (N - np.arange(N)))) * per_u  # u channel: on u_i
-    if nc != 16:                                               # (the TRI kernel sums in place)
-        tot += (N * N * (N + 1) / 2) * P * nc                  # lattice-sum gather per triple
     return tot
 
 
 def _kernel_hash() -> str:
-    """Hash of the device code of the vertex kernels: kernels.cuh, tc.cuh, su2f.cuh and flow.cu
+    """Hash of the device code of the vertex kernels: kernels.cuh, tc.cuh, pair.cuh and flow.cu
     up to its host-side objects (changes to host code leave committed ncu figures valid)."""
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2109_13317_gb300", "csrc")
-    for f in ("kernels.cuh", "tc.cuh", "su2f.cuh"):
+    for f in ("kernels.cuh", "tc.cuh", "pair.cuh"):
         with open(os.path.join(csrc, f), "rb") as fh:
             h.update(fh.read())
     with open(os.path.join(csrc, "flow.cu"), "rb") as fh:
         src = fh.read()
-    h.update(src.split(b'#include "adjoint.cuh"')[0])
+    h.update(src.split(b'#include "chi.cuh"')[0])
     return h.hexdigest()[:16]
 
 
@@ -605,7 +611,7 @@ def run_ours(args):
     value = _job_throughput(n_ent, ws, t_step)
 
     # roofline of the dominant kernel (vertex flow)
-    flops = _algorithmic_flops(counts, fl.N, lat.N_s, fl.n_comp, lat.P, fl.lattice_sum_products())
+    flops = _algorithmic_flops(counts, fl.N, lat.N_s, fl.n_comp, lat.P, fl.lattice_sum_products(), _graded(cfg.model))
     k_ms = kms[2] / max(kn[2], 1)
     achieved = flops / (k_ms * 1e-3) / 1e12
     peak_fp64_nominal = 1.25     # TFLOP/s, recipe table
@@ -623,7 +629,7 @@ def run_ours(args):
         ck32, _ = fl2.measure(kgrid, want_ij=False)
         _, G64 = fl.get_state()
         _, G32 = fl2.get_state()
-        flops2 = _algorithmic_flops(counts2, fl2.N, lat.N_s, fl2.n_comp, lat.P, fl2.lattice_sum_products())
+        flops2 = _algorithmic_flops(counts2, fl2.N, lat.N_s, fl2.n_comp, lat.P, fl2.lattice_sum_products(), _graded(cfg.model))
         k2 = kms2[2] / max(kn2[2], 1)
         tcv = _tensor_core_variant(sr, torch, fl2)
         extra["fp32_mixed"] = {"value": n_ent * ws / (sum(ms2) / len(ms2) * 1e-3), "unit": UNIT,
@@ -722,7 +728,7 @@ def run_ours(args):
                        "lambda_range_timed": [float(lam_rng[0]), float(lam_rng[1])],
                        "l2": "flushed between timed steps (256 MB write)",
                        "parallelism": f"replicas x{ws}" if ws > 1 else "single GPU"},
-            "roofline": {"bound": "alu", "kernel": "k_gamma_rhs_tri" if fl.n_comp == 16 else "k_gamma_rhs",
+            "roofline": {"bound": "alu", "kernel": "k_gamma_rhs_trid" if fl.n_comp == 16 else "k_gamma_rhs_pair",
                          "achieved": achieved, "peak": peak,
                          "unit": "TFLOP/s", "frac": achieved / peak,
                          "peak_source": "FP64 nominal 1.25 TFLOP/s (recipe table)" if prec == sr.SR_FP64 else

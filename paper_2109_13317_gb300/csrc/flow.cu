@@ -1405,6 +1405,20 @@ struct DevBuf {
     }
 };
 
+// Small host tables that go to the device in one allocation and one copy.
+struct TableBlob {
+    std::vector<unsigned char> bytes;
+    template <typename T>
+    size_t add(const std::vector<T>& v) { return add(v.data(), v.size()); }
+    template <typename T>
+    size_t add(const T* v, size_t n) {   // v null: zeros
+        const size_t o = (bytes.size() + 15) & ~size_t(15);
+        bytes.resize(o + sizeof(T) * std::max<size_t>(n, 1), 0);
+        if (v && n) memcpy(bytes.data() + o, v, sizeof(T) * n);
+        return o;
+    }
+};
+
 struct sr_flow {
     const sr_lattice* lat = nullptr;
     Geo g{};
@@ -1438,8 +1452,12 @@ struct sr_flow {
     DevBuf<int> chi_onsite;
     DevBuf<double> chi_dr, chi, kbuf, chik;
     // correlations of the SU2 / XYZ cores (chik::): displacements merged up to sign, partial sums
-    DevBuf<double> chi_d, chi_sd, chi_part;
-    DevBuf<int> chi_doff, chi_dpair, chi_counter;
+    DevBuf<unsigned char> chi_tables;
+    DevBuf<double> chi_part;
+    const double* chi_d = nullptr;
+    double* chi_sd = nullptr;
+    const int *chi_doff = nullptr, *chi_dpair = nullptr;
+    int* chi_counter = nullptr;
     int chi_nd = 0;
     DevBuf<int> flag;             // [0] non-finite value, [1] the tensor-core kernel's MMA wait gave up
     DevBuf<unsigned long long> errbits;
@@ -1479,19 +1497,15 @@ struct sr_flow {
     pairk::Tab pk{};
     int pk_variant = -1, pk_threads = 0;
     size_t pk_smem = 0;
-    DevBuf<int> pk_terms, pk_n_terms, pk_kap;
-    DevBuf<int2> pk_prod;
-    DevBuf<double> pk_mult;
+    DevBuf<unsigned char> pk_tables;
     // TRI vertex flow with the dense lattice sum (trid::): tables, packed state, and the flag that
     // sends a state with odd components to the general kernel (graded lattices)
     trid::Tab td{};
     trid::Choice<float> tdf;
     trid::Choice<double> tdd;
     bool td_on = false, td_graded = false;
-    DevBuf<int2> td_pack;
-    DevBuf<unsigned> td_fmap;
-    DevBuf<int> td_ent, td_run_pair, td_n_terms, td_terms, td_flag;
-    DevBuf<int2> td_runs;
+    DevBuf<unsigned char> td_tables;
+    int* td_flag = nullptr;
     DevBuf<float> Pf;
     DevBuf<double> Pd;
 
@@ -1591,18 +1605,18 @@ static void launch_gamma_tri(sr_flow* f, const double* G_s, const float* Gf_s, d
     if (f->td_on) {
         const unsigned pblocks = (unsigned)std::min<long>((long)g.npair * g.N, 4096);
         if (f->td_graded) {
-            use = f->td_flag.p;
-            cudaMemsetAsync(f->td_flag.p, 0, sizeof(int), st);
+            use = f->td_flag;
+            cudaMemsetAsync(f->td_flag, 0, sizeof(int), st);
         }
         if (f->prec == SR_FP64) {
-            if (f->td_graded) trid::k_tri_pack<double, true><<<pblocks, 128, 0, st>>>(g, f->td, G_s, f->Pd.p, f->td_flag.p);
+            if (f->td_graded) trid::k_tri_pack<double, true><<<pblocks, 128, 0, st>>>(g, f->td, G_s, f->Pd.p, f->td_flag);
             else trid::k_tri_pack<double, false><<<pblocks, 128, 0, st>>>(g, f->td, G_s, f->Pd.p, nullptr);
             f->tdd.fn<<<blocks, f->tdd.threads, f->tdd.smem, st>>>(g, tb, f->td, f->w.p, f->Pd.p, f->nx.p, f->nW.p, f->ncount.p,
                                                                    dG_o, pb, use, 0);
         } else {
             if (f->td_graded) {
-                trid::k_tri_pack<float, true><<<pblocks, 128, 0, st>>>(g, f->td, G_s, f->Pf.p, f->td_flag.p);
-                trid::k_shadow_if<<<1024, 256, 0, st>>>(g.nent, G_s, f->Gf.p, f->td_flag.p);
+                trid::k_tri_pack<float, true><<<pblocks, 128, 0, st>>>(g, f->td, G_s, f->Pf.p, f->td_flag);
+                trid::k_shadow_if<<<1024, 256, 0, st>>>(g.nent, G_s, f->Gf.p, f->td_flag);
             } else {
                 trid::k_tri_pack<float, false><<<pblocks, 128, 0, st>>>(g, f->td, G_s, f->Pf.p, nullptr);
             }
@@ -1916,16 +1930,16 @@ static sr_status flow_create(const sr_lattice* lat, int n_freq, const double* fr
             f->pk_variant = pl.variant;
             f->pk_threads = pl.threads;
             f->pk_smem = pl.smem;
-            CK(f->pk_terms.upload(pl.terms.data(), pl.terms.size(), f->stream));
-            CK(f->pk_n_terms.upload(pl.n_terms.data(), pl.n_terms.size(), f->stream));
-            CK(f->pk_prod.upload(pl.prod.data(), pl.prod.size(), f->stream));
-            CK(f->pk_kap.upload(pl.kap.data(), pl.kap.size(), f->stream));
-            CK(f->pk_mult.upload(pl.mult.data(), pl.mult.size(), f->stream));
-            f->pk.kap = f->pk_kap.p;
-            f->pk.mult = f->pk_mult.p;
-            f->pk.terms = f->pk_terms.p;
-            f->pk.n_terms = f->pk_n_terms.p;
-            f->pk.prod = f->pk_prod.p;
+            TableBlob tbl;
+            const size_t o_terms = tbl.add(pl.terms), o_n = tbl.add(pl.n_terms), o_prod = tbl.add(pl.prod), o_kap = tbl.add(pl.kap),
+                         o_mult = tbl.add(pl.mult);
+            CK(f->pk_tables.upload(tbl.bytes.data(), tbl.bytes.size(), f->stream));
+            unsigned char* base = f->pk_tables.p;
+            f->pk.terms = (const int*)(base + o_terms);
+            f->pk.n_terms = (const int*)(base + o_n);
+            f->pk.prod = (const int2*)(base + o_prod);
+            f->pk.kap = (const int*)(base + o_kap);
+            f->pk.mult = (const double*)(base + o_mult);
             const size_t np = (size_t)pl.size;
             if (precision == SR_FP64) {
                 CK(f->Pd.alloc(np));
@@ -1970,13 +1984,17 @@ static sr_status flow_create(const sr_lattice* lat, int n_freq, const double* fr
         if (g.nc != 16 && !f->ntan) {
             const chik::Displacements D = chik::merge(lat->chi_dr);
             f->chi_nd = (int)D.off.size() - 1;
-            CK(f->chi_d.upload(D.dr.data(), D.dr.size(), st));
-            CK(f->chi_doff.upload(D.off.data(), D.off.size(), st));
-            CK(f->chi_dpair.upload(D.pair.data(), D.pair.size(), st));
-            CK(f->chi_sd.alloc(f->chi_nd));
+            TableBlob tbl;
+            const size_t o_d = tbl.add(D.dr), o_off = tbl.add(D.off), o_pair = tbl.add(D.pair),
+                         o_sd = tbl.add<double>(nullptr, f->chi_nd), o_cnt = tbl.add<int>(nullptr, 1);
+            CK(f->chi_tables.upload(tbl.bytes.data(), tbl.bytes.size(), st));
+            unsigned char* base = f->chi_tables.p;
+            f->chi_d = (const double*)(base + o_d);
+            f->chi_doff = (const int*)(base + o_off);
+            f->chi_dpair = (const int*)(base + o_pair);
+            f->chi_sd = (double*)(base + o_sd);
+            f->chi_counter = (int*)(base + o_cnt);   // zero between launches
             CK(f->chi_part.alloc(chik::part_doubles(g.Ns, g.nc)));
-            CK(f->chi_counter.alloc(1));
-            CK(cudaMemsetAsync(f->chi_counter.p, 0, sizeof(int), st));
             const size_t sm = sizeof(double) * 2 * g.Ns * g.nc * chik::groups(g.Ns * g.nc);
             if (sm > 32 * 1024) CK(ensure_smem(g.nc == 2 ? (const void*)chik::k_chi_sum<2> : (const void*)chik::k_chi_sum<4>, sm));
         }
@@ -2083,17 +2101,17 @@ static sr_status flow_create(const sr_lattice* lat, int n_freq, const double* fr
             if (on) {
                 f->td_on = true;
                 f->td_graded = pl.graded;
-                CK(f->td_pack.upload(pl.pack.data(), pl.pack.size(), st));
-                CK(f->td_fmap.upload(pl.fmap.data(), pl.fmap.size(), st));
-                CK(f->td_ent.upload(pl.ent.data(), pl.ent.size(), st));
-                CK(f->td_runs.upload(pl.runs.data(), pl.runs.size(), st));
-                CK(f->td_run_pair.upload(pl.run_pair.data(), pl.run_pair.size(), st));
-                CK(f->td_n_terms.upload(pl.n_terms.data(), pl.n_terms.size(), st));
-                CK(f->td_terms.upload(pl.terms.data(), pl.terms.size(), st));
-                CK(f->td_flag.alloc(1));
+                TableBlob tbl;
+                const size_t o_pack = tbl.add(pl.pack), o_fmap = tbl.add(pl.fmap), o_ent = tbl.add(pl.ent), o_runs = tbl.add(pl.runs),
+                             o_pair = tbl.add(pl.run_pair), o_n = tbl.add(pl.n_terms), o_terms = tbl.add(pl.terms),
+                             o_flag = tbl.add<int>(nullptr, 1);
+                CK(f->td_tables.upload(tbl.bytes.data(), tbl.bytes.size(), st));
+                unsigned char* base = f->td_tables.p;
+                f->td_flag = (int*)(base + o_flag);
                 trid::Tab& td = f->td;
-                td.pack = f->td_pack.p; td.fmap = f->td_fmap.p; td.ent = f->td_ent.p; td.runs = f->td_runs.p;
-                td.run_pair = f->td_run_pair.p; td.n_terms = f->td_n_terms.p; td.terms = f->td_terms.p;
+                td.pack = (const int2*)(base + o_pack); td.fmap = (const unsigned*)(base + o_fmap); td.ent = (const int*)(base + o_ent);
+                td.runs = (const int2*)(base + o_runs); td.run_pair = (const int*)(base + o_pair);
+                td.n_terms = (const int*)(base + o_n); td.terms = (const int*)(base + o_terms);
                 td.n_runs = (int)pl.runs.size(); td.nk = pl.nk;
                 for (int k = 0; k < trid::kMaxPairs; ++k) td.kap[k] = pl.kap[k];
                 for (int k = 0; k < 4; ++k) td.spin[k] = pl.spin[k];
@@ -2505,12 +2523,12 @@ static void launch_chi(sr_flow* f, double* chi) {
     const size_t sm = sizeof(double) * 2 * g.Ns * g.nc * chik::groups(g.Ns * g.nc);
     if (g.nc == 2)
         chik::k_chi_sum<2><<<nb, chik::kThreads, sm, f->stream>>>(g, tb, f->w.p, f->gam.p, f->G.p, f->lambda, f->chi_map.p, f->chi_onsite.p,
-                                                                  f->lat->Ntot, npairs, f->chi_doff.p, f->chi_dpair.p, f->chi_nd,
-                                                                  f->chi_part.p, f->chi_counter.p, chi, f->chi_sd.p);
+                                                                  f->lat->Ntot, npairs, f->chi_doff, f->chi_dpair, f->chi_nd,
+                                                                  f->chi_part.p, f->chi_counter, chi, f->chi_sd);
     else
         chik::k_chi_sum<4><<<nb, chik::kThreads, sm, f->stream>>>(g, tb, f->w.p, f->gam.p, f->G.p, f->lambda, f->chi_map.p, f->chi_onsite.p,
-                                                                  f->lat->Ntot, npairs, f->chi_doff.p, f->chi_dpair.p, f->chi_nd,
-                                                                  f->chi_part.p, f->chi_counter.p, chi, f->chi_sd.p);
+                                                                  f->lat->Ntot, npairs, f->chi_doff, f->chi_dpair, f->chi_nd,
+                                                                  f->chi_part.p, f->chi_counter, chi, f->chi_sd);
 }
 
 extern "C" sr_status sr_measure_susceptibility(sr_flow* f, int n_k, const double* k_xyz, double* chi_k, double* chi_ij) {
@@ -2535,7 +2553,7 @@ extern "C" sr_status sr_measure_susceptibility(sr_flow* f, int n_k, const double
         if (g.nc == 16)
             k_chi_k_tri<<<(n_k + 127) / 128, 128, 0, f->stream>>>(n_k, f->kbuf.p, f->chi.p, f->chi_dr.p, npairs, lat->nb, f->chik.p);
         else
-            chik::k_chi_fourier<<<(n_k + 3) / 4, chik::kThreads, 0, f->stream>>>(n_k, f->kbuf.p, f->chi_d.p, f->chi_sd.p, f->chi_nd, lat->nb, f->chik.p);
+            chik::k_chi_fourier<<<(n_k + 3) / 4, chik::kThreads, 0, f->stream>>>(n_k, f->kbuf.p, f->chi_d, f->chi_sd, f->chi_nd, lat->nb, f->chik.p);
         CK(cudaGetLastError());
         CK(cudaMemcpyAsync(chi_k, f->chik.p, sizeof(double) * n_k, cudaMemcpyDeviceToHost, f->stream));
         CK(cudaStreamSynchronize(f->stream));
@@ -3600,7 +3618,7 @@ extern "C" sr_status sr_measure_susceptibility_static(sr_flow* f, int n_k, const
         if (g.nc == 16)
             k_chi_k_tri<<<(n_k + 127) / 128, 128, 0, f->stream>>>(n_k, d_k_xyz, scratch, f->chi_dr.p, npairs, lat->nb, d_chi_k);
         else
-            chik::k_chi_fourier<<<(n_k + 3) / 4, chik::kThreads, 0, f->stream>>>(n_k, d_k_xyz, f->chi_d.p, f->chi_sd.p, f->chi_nd, lat->nb, d_chi_k);
+            chik::k_chi_fourier<<<(n_k + 3) / 4, chik::kThreads, 0, f->stream>>>(n_k, d_k_xyz, f->chi_d, f->chi_sd, f->chi_nd, lat->nb, d_chi_k);
         CK(cudaGetLastError());
     }
     return SR_OK;

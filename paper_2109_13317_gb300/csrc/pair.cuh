@@ -19,9 +19,9 @@
 // a node needs four interval searches per channel for its two to four rows.
 //
 // Measured (vertex kernel, one GB300; before: the general FP64 kernel and the FP32 kernels on
-// component rows): square J1-J2 range 7, 48 frequencies, FP64 13.2 -> 11.8 ms, FP32 1.55 -> 0.98 ms;
-// pyrochlore range 6, 64 frequencies, FP32 12.6 -> 8.0 ms; honeycomb Heisenberg-Kitaev range 5,
-// 32 frequencies, FP64 3.65 -> 2.95 ms, FP32 0.60 -> 0.40 ms.
+// component rows): square J1-J2 range 7, 48 frequencies, FP64 13.2 -> 10.5 ms, FP32 1.55 -> 0.98 ms;
+// pyrochlore range 6, 64 frequencies, FP32 12.6 -> 7.9 ms; honeycomb Heisenberg-Kitaev range 5,
+// 32 frequencies, FP64 3.65 -> 2.85 ms, FP32 0.60 -> 0.35 ms.
 // What bounds it: FP64, the FP64 pipe (92 % busy on the square lattice); FP32, the L1 data path (86 %
 // busy there: a corner chunk is one 16-byte load per 4 multiply-adds, and a row of 160 bytes touches
 // two 128-byte lines).  Tried and dropped in FP32: corner chunks kept in registers over a run of
@@ -481,18 +481,39 @@ __device__ __forceinline__ void triple(const Geo& g, const Tabs& tb, const Tab& 
     }
     if (in_stream) st16(tt + (2 * stream + rw) * rt + ct * V, pt);
     __syncthreads();
-    for (int o = tid; o < NC * Ns; o += nth) {
-        const int c = o / Ns, r = o - c * Ns;
-        R es[NC], eu[NC], a = R(0), l = R(0);
-#pragma unroll
-        for (int e = 0; e < NC; ++e) {
-            es[e] = eu[e] = R(0);
-            for (int k = 0; k < NG; ++k) {
-                es[e] += su[(2 * k) * rv + e * Ns + r];
-                eu[e] += su[(2 * k + 1) * rv + e * Ns + r];
+    // FP64 and long rows: the sums over groups and streams first, a value each (into the slots of the
+    // first group and stream), instead of every output summing all eigenvalues it mixes (square range 7
+    // FP64 11.85 -> 11.70 ms, pyrochlore FP32 8.39 -> 8.18; the short FP32 rows lose 3 % by the barrier)
+    constexpr bool kStage = sizeof(R) == 8 || TM == 8;
+    if constexpr (kStage) {
+        for (int v = tid; v < 2 * rv + rt; v += nth) {
+            if (v < 2 * rv) {
+                R a = su[v];
+                for (int k = 1; k < NG; ++k) a += su[2 * k * rv + v];
+                su[v] = a;
+            } else {
+                R a = tt[v - 2 * rv];
+                for (int k = 1; k < 2 * S; ++k) a += tt[k * rt + v - 2 * rv];
+                tt[v - 2 * rv] = a;
             }
         }
-        for (int k = 0; k < 2 * S; ++k) a += tt[k * rt + c * nst + r];
+        __syncthreads();
+    }
+    for (int o = tid; o < NC * Ns; o += nth) {
+        const int c = o / Ns, r = o - c * Ns;
+        R es[NC], eu[NC], a = tt[c * nst + r], l = R(0);
+#pragma unroll
+        for (int e = 0; e < NC; ++e) {
+            es[e] = su[e * Ns + r];
+            eu[e] = su[rv + e * Ns + r];
+            if constexpr (!kStage)
+                for (int k = 1; k < NG; ++k) {
+                    es[e] += su[(2 * k) * rv + e * Ns + r];
+                    eu[e] += su[(2 * k + 1) * rv + e * Ns + r];
+                }
+        }
+        if constexpr (!kStage)
+            for (int k = 1; k < 2 * S; ++k) a += tt[k * rt + c * nst + r];
         const int nt = td.n_terms[r];
 #pragma unroll 4
         for (int k = 0; k < nt; ++k) {
@@ -620,7 +641,8 @@ using Kernel = void (*)(Geo, Tabs, Tab, const R*, const R*, const R*, const int*
 // multiple the sites of a t row are padded to).  FP32 tiles of 8 x 4 instead of 4 x 4 save
 // operand loads once the rows are long (pyrochlore: one tile on 160 threads 8.0 ms, two on 96 9.7 ms);
 // up to 20 sites 4 x 4 tiles fill 64 threads.  FP64 lists have no padding, tiles take over where the
-// products exceed eight per thread.
+// products exceed eight per thread; their registers are capped for six CTAs of 128 threads (square range
+// 7: five 11.7 ms, six 10.5, seven and eight 10.5; 13 products on 64 threads 11.3; 160 threads 12.8).
 #define PAIR_F32_VARIANTS(X)     \
     X(0, 2, 4, 4, 1, 64, 12, 4)  \
     X(1, 2, 8, 4, 1, 160, 5, 8)  \
@@ -630,8 +652,8 @@ using Kernel = void (*)(Geo, Tabs, Tab, const R*, const R*, const R*, const int*
     X(5, 4, 4, 4, 2, 192, 3, 4)  \
     X(6, 4, 4, 4, 4, 384, 1, 4)
 #define PAIR_F64_VARIANTS(X)     \
-    X(0, 2, 1, 1, 2, 64, 10, 2)  \
-    X(1, 2, 1, 1, 8, 128, 5, 2)  \
+    X(0, 2, 1, 1, 2, 64, 12, 2)  \
+    X(1, 2, 1, 1, 8, 128, 6, 2)  \
     X(2, 2, 2, 2, 5, 256, 2, 2)  \
     X(3, 2, 2, 2, 10, 256, 2, 2) \
     X(4, 4, 1, 1, 2, 64, 10, 2)  \

@@ -13,10 +13,10 @@
 //   * the transposed lookups add to accumulators in the packed layout (both eigenvalue tables, the
 //     component rows, and the same of the exchanged pairs), so lanes add to consecutive addresses;
 //     k_pair_fold maps them onto the state.
-// Heisenberg-Kitaev, range 5, 32 frequencies (one GB300): 15.8 -> 9.9 ms.  The FP64 pipe still bounds
+// Heisenberg-Kitaev, range 5, 32 frequencies (one GB300): 15.8 -> 9.7 ms.  The FP64 pipe still bounds
 // it (81 % busy): 8 + 8 operations per value and node for the interpolation and its transpose, two per
 // product and node for the lattice sum.  Lists sorted by length (a warp runs as long as its longest):
-// 10.8 -> 9.9.
+// 10.8 -> 9.9; registers capped for six CTAs instead of four: 9.9 -> 9.7.
 #pragma once
 
 namespace pairk {
@@ -62,7 +62,7 @@ __device__ __forceinline__ void red2(double* p, double w, const double* v) {
 // Abar += (d dGamma / d Gamma)^T fbar in the packed layout, Wbar += d dGamma / d W . fbar; one CTA per
 // stored triple.
 template <int NC>
-__global__ void __launch_bounds__(128, 4)
+__global__ void __launch_bounds__(128, 6)
 k_gamma_adj_pair(Geo g, Tabs tb, Tab td, AdjTab at, const double* __restrict__ P, const double* __restrict__ nx,
                  const double* __restrict__ nW, const int* __restrict__ ncount, const double* __restrict__ fbar,
                  double* __restrict__ Pbar, double* __restrict__ Wbar) {
