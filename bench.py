@@ -714,7 +714,8 @@ def run_ours(args):
         except Exception as e:  # the oracle is a baseline, never the product path
             cpu = {"value": None, "unit": UNIT, "cores": None, "kind": "oracle", "sample": f"failed: {e}"}
 
-    launches_per_step = 5 + 1 + (1 if prec == sr.SR_FP32_MIXED else 0)  # sigma, nodes, gamma, 2 axpy, chi (+1 shadow)
+    # sigma, nodes, pack, gamma, update, chi_ij, chi(k) (the general core launches one or two more)
+    launches_per_step = 7
     if rank == 0:
         line = {
             "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": ws, "steps": args.steps,

@@ -8,11 +8,15 @@
 //                      nodes and weights -- four exact delta points of S and the trapezoid
 //                      rule on the regular Katanin part -- shared by every vertex entry
 //                      with that transfer frequency (the paper's buffered weights).
-//   3. k_gamma_rhs     one CTA per stored (s, u, t) triple: all sites and components.
-//                      Per block of integration nodes it builds the interpolated vertex
-//                      rows over all irreducible sites in shared memory, then the s / u
-//                      channel products, the t-channel on-site terms, and the lattice sum
-//                      sum_j Gamma_{i1 j} Gamma_{j i2} through the tabulated site list.
+//   3. the vertex flow on packed interpolation rows: k_pair_pack / k_gamma_rhs_pair
+//                      (SU2, XYZ: pair.cuh), k_tri_pack / k_gamma_rhs_trid (general core:
+//                      tri_dense.cuh).  One CTA per stored (s, u, t) triple: all sites and
+//                      components; per block of integration nodes the interpolated rows,
+//                      the s / u channel products, the t-channel on-site terms and the
+//                      lattice sum sum_j Gamma_{i1 j} Gamma_{j i2} through the tabulated
+//                      site list.  k_gamma_rhs / k_gamma_rhs_f32 / k_gamma_rhs_tri below do
+//                      the same from the stored state, for tangent flows (dual numbers) and
+//                      for lattices whose rows or tables do not fit the packed plans.
 #include <cuda_runtime.h>
 
 #include <algorithm>
