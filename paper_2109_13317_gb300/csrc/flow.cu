@@ -1847,6 +1847,7 @@ static sr_status flow_create(const sr_lattice* lat, int n_freq, const double* fr
     f->ntan = npar > 0 ? kTan : 0;
     f->ts = 1 + f->ntan;
     const int ts = f->ts;
+    size_t n_packed = 0;   // values of the packed state
     std::vector<double> init_host = lat->init_gamma;
     if (npar > 0) {
         std::vector<double> dinit;
@@ -1944,16 +1945,9 @@ static sr_status flow_create(const sr_lattice* lat, int n_freq, const double* fr
             f->pk.prod = (const int2*)(base + o_prod);
             f->pk.kap = (const int*)(base + o_kap);
             f->pk.mult = (const double*)(base + o_mult);
-            const size_t np = (size_t)pl.size;
-            if (precision == SR_FP64) {
-                CK(f->Pd.alloc(np));
-                CK(cudaMemsetAsync(f->Pd.p, 0, sizeof(double) * np, f->stream));   // padding stays zero
-                CK(ensure_smem((const void*)pairk::kernel_f64(pl.variant), pl.smem));
-            } else {
-                CK(f->Pf.alloc(np));
-                CK(cudaMemsetAsync(f->Pf.p, 0, sizeof(float) * np, f->stream));
-                CK(ensure_smem((const void*)pairk::kernel_f32(pl.variant), pl.smem));
-            }
+            n_packed = (size_t)pl.size;
+            CK(ensure_smem(precision == SR_FP64 ? (const void*)pairk::kernel_f64(pl.variant) : (const void*)pairk::kernel_f32(pl.variant),
+                           pl.smem));
         }
     }
     std::vector<double> ih(n_freq - 1);
@@ -2122,9 +2116,7 @@ static sr_status flow_create(const sr_lattice* lat, int n_freq, const double* fr
                 td.nrow = (int)nrow;
                 const unsigned long long half = (unsigned long long)(pl.graded ? Ns : 2 * Ns);
                 td.div_half = half > 1 ? (unsigned)((0x100000000ULL + half - 1) / half) : 0u;
-                const size_t np = (size_t)g.nent * (pl.graded ? 1 : 2);
-                if (precision == SR_FP64) CK(f->Pd.alloc(np));
-                else CK(f->Pf.alloc(np));
+                n_packed = (size_t)g.nent * (pl.graded ? 1 : 2);
             }
         }
     }
@@ -2133,6 +2125,19 @@ static sr_status flow_create(const sr_lattice* lat, int n_freq, const double* fr
     CK(f->G.alloc((size_t)g.nent * ts));
     CK(f->dgam.alloc((size_t)g.N * ts));
     CK(f->dG.alloc((size_t)g.nent * ts));
+    if (n_packed > 0) {   // where it finds no memory the kernels on the stored state serve the flow
+        const cudaError_t e = precision == SR_FP64 ? f->Pd.alloc(n_packed) : f->Pf.alloc(n_packed);
+        if (e == cudaErrorMemoryAllocation) {
+            cudaGetLastError();
+            f->Pd.p = nullptr;
+            f->Pf.p = nullptr;
+            f->pk_on = f->td_on = false;
+        } else {
+            CK(e);
+            if (f->Pd.p && f->pk_on) CK(cudaMemsetAsync(f->Pd.p, 0, sizeof(double) * n_packed, st));   // padding stays zero
+            if (f->Pf.p && f->pk_on) CK(cudaMemsetAsync(f->Pf.p, 0, sizeof(float) * n_packed, st));
+        }
+    }
     if (precision == SR_FP32_MIXED && !(f->td_on && !f->td_graded) && !f->pk_on)
         CK(f->Gf.alloc(g.nc == 16 ? (size_t)g.nent : (size_t)g.nentp * (f->has_swap ? 2 : 1)));
     CK(f->nx.alloc((size_t)3 * g.N * g.nmax));
