@@ -1395,9 +1395,12 @@ template <typename T>
 struct DevBuf {
     T* p = nullptr;
     size_t n = 0;
-    ~DevBuf() { if (p) cudaFree(p); }
+    bool view = false;   // part of a TableSet: not freed here
+    ~DevBuf() { if (p && !view) cudaFree(p); }
     cudaError_t alloc(size_t count) {
-        if (p) { cudaFree(p); p = nullptr; }
+        if (p && !view) cudaFree(p);
+        p = nullptr;
+        view = false;
         n = count;
         if (count == 0) return cudaSuccess;
         return cudaMalloc((void**)&p, sizeof(T) * count);
@@ -1423,6 +1426,30 @@ struct TableBlob {
     }
 };
 
+// Tables of a flow that share one allocation and one copy (each of its own costs an allocation,
+// a copy and a call to free them: a tenth of a small flow's creation).
+struct TableSet {
+    TableBlob tbl;
+    std::vector<std::pair<void*, size_t>> at;   // address of the buffer's pointer, offset
+    template <typename T>
+    void add(DevBuf<T>& d, const T* v, size_t n) {
+        d.alloc(0);
+        d.n = n;
+        if (n == 0) return;
+        d.view = true;
+        at.emplace_back(&d.p, tbl.add(v, n));
+    }
+    cudaError_t upload(DevBuf<unsigned char>& base, cudaStream_t st) {
+        const cudaError_t e = base.upload(tbl.bytes.data(), tbl.bytes.size(), st);
+        if (e != cudaSuccess) return e;
+        for (const auto& x : at) {
+            const void* q = base.p + x.second;
+            memcpy(x.first, &q, sizeof(q));
+        }
+        return e;
+    }
+};
+
 struct sr_flow {
     const sr_lattice* lat = nullptr;
     Geo g{};
@@ -1434,6 +1461,7 @@ struct sr_flow {
     int ntan = 0;   // tangent directions (0: plain flow; kTan: the state holds Dual<kTan> values)
     int ts = 1;     // doubles per state scalar
 
+    DevBuf<unsigned char> tables;   // of the buffers that flow_create adds to its TableSet
     DevBuf<double> w, gam, G, dgam, dG;
     DevBuf<float> Gf;
     DevBuf<double> nx, nW;
@@ -1848,6 +1876,7 @@ static sr_status flow_create(const sr_lattice* lat, int n_freq, const double* fr
     f->ts = 1 + f->ntan;
     const int ts = f->ts;
     size_t n_packed = 0;   // values of the packed state
+    TableSet tabs;
     std::vector<double> init_host = lat->init_gamma;
     if (npar > 0) {
         std::vector<double> dinit;
@@ -1884,19 +1913,20 @@ static sr_status flow_create(const sr_lattice* lat, int n_freq, const double* fr
     std::vector<int2> prods;
     std::vector<int> goff(lat->Ns * lat->nc + 1, 0), gidx;
     if (lat->nc != 16) {
-        std::map<std::pair<int, int>, int> pid;
+        size_t cap = 16;   // open addressing, numbered by first occurrence: the search of a tree took
+        while (cap < 2 * lat->rpa.size() * lat->nc) cap *= 2;   // a tenth of a flow's creation
+        std::vector<int> slot(cap, -1);
+        gidx.reserve(lat->rpa.size() * lat->nc);
         for (int r = 0; r < lat->Ns; ++r)
             for (int c = 0; c < lat->nc; ++c) {
                 goff[r * lat->nc + c] = (int)gidx.size();
                 for (int e = lat->rpa_off[r]; e < lat->rpa_off[r + 1]; ++e) {
                     const sr::RpaEntry& en = lat->rpa[e];
                     int ia = en.rA * lat->nc + en.pA[c], ib = en.rB * lat->nc + en.pB[c];
-                    auto key = std::make_pair(ia, ib);
-                    auto it = pid.find(key);
-                    int u;
-                    if (it == pid.end()) { u = (int)prods.size(); pid[key] = u; prods.push_back(make_int2(ia, ib)); }
-                    else u = it->second;
-                    gidx.push_back(u);
+                    size_t h = (((unsigned long long)ia << 32 | (unsigned)ib) * 0x9E3779B97F4A7C15ULL >> 32) & (cap - 1);
+                    while (slot[h] >= 0 && (prods[slot[h]].x != ia || prods[slot[h]].y != ib)) h = (h + 1) & (cap - 1);
+                    if (slot[h] < 0) { slot[h] = (int)prods.size(); prods.push_back(make_int2(ia, ib)); }
+                    gidx.push_back(slot[h]);
                 }
             }
         goff[lat->Ns * lat->nc] = (int)gidx.size();
@@ -1914,7 +1944,7 @@ static sr_status flow_create(const sr_lattice* lat, int n_freq, const double* fr
             const int rb = prods[k].y / lat->nc, cb = prods[k].y % lat->nc;
             pp[k] = make_int2(ca * nsp + ra, cb * nsp + rb);
         }
-        CK(f->prodp.upload(pp.data(), pp.size(), f->stream));
+        tabs.add(f->prodp, pp.data(), pp.size());
         f->has_swap = false;
         for (int r = 0; r < lat->Ns; ++r) {
             if (lat->swap_r[r] != r) f->has_swap = true;
@@ -1927,7 +1957,7 @@ static sr_status flow_create(const sr_lattice* lat, int n_freq, const double* fr
             const int rb = prods[gidx[k]].y / lat->nc;
             dg[k] = ca * nsp * nsp + ra * nsp + rb;
         }
-        CK(f->dgath_idx.upload(dg.data(), dg.size(), f->stream));
+        tabs.add(f->dgath_idx, dg.data(), dg.size());
         pairk::Plan pl;
         if (!f->ntan && pairk::build_plan(lat, n_freq, precision != SR_FP64, f->has_swap, prods, goff, gidx, &pl)) {
             f->pk_on = true;
@@ -1953,31 +1983,31 @@ static sr_status flow_create(const sr_lattice* lat, int n_freq, const double* fr
     std::vector<double> ih(n_freq - 1);
     for (int i = 0; i + 1 < n_freq; ++i) ih[i] = 1.0 / (freq_pos[i + 1] - freq_pos[i]);
     cudaStream_t st = f->stream;
-    CK(f->w.upload(freq_pos, n_freq, st));
-    CK(f->invh.upload(ih.data(), ih.size(), st));
+    tabs.add(f->w, freq_pos, n_freq);
+    tabs.add(f->invh, ih.data(), ih.size());
     {
         std::vector<float> wfl(n_freq), ihf(n_freq - 1);
         for (int i = 0; i < n_freq; ++i) wfl[i] = (float)freq_pos[i];
         for (int i = 0; i + 1 < n_freq; ++i) ihf[i] = 1.0f / (wfl[i + 1] - wfl[i]);
-        CK(f->wf.upload(wfl.data(), wfl.size(), st));
-        CK(f->invhf.upload(ihf.data(), ihf.size(), st));
+        tabs.add(f->wf, wfl.data(), wfl.size());
+        tabs.add(f->invhf, ihf.data(), ihf.size());
         g.log2w0 = (float)std::log2(freq_pos[0]);
         g.inv_dlog2 = (float)((n_freq - 1) / std::log2(freq_pos[n_freq - 1] / freq_pos[0]));
     }
-    CK(f->swap_r.upload(lat->swap_r.data(), lat->Ns, st));
-    CK(f->swap_perm.upload(sp.data(), lat->Ns, st));
-    CK(f->onsite_perm.upload(op.data(), lat->Ns, st));
-    CK(f->mult.upload(lat->mult.data(), lat->Ns, st));
-    CK(f->prod.upload(prods.data(), prods.size(), st));
-    CK(f->gath_off.upload(goff.data(), goff.size(), st));
-    CK(f->gath_idx.upload(gidx.data(), gidx.size(), st));
-    CK(f->init.upload(init_host.data(), init_host.size(), st));
+    tabs.add(f->swap_r, lat->swap_r.data(), lat->Ns);
+    tabs.add(f->swap_perm, sp.data(), lat->Ns);
+    tabs.add(f->onsite_perm, op.data(), lat->Ns);
+    tabs.add(f->mult, lat->mult.data(), lat->Ns);
+    tabs.add(f->prod, prods.data(), prods.size());
+    tabs.add(f->gath_off, goff.data(), goff.size());
+    tabs.add(f->gath_idx, gidx.data(), gidx.size());
+    tabs.add(f->init, init_host.data(), init_host.size());
     {
         std::vector<int2> cm(lat->chi_map.size());
         for (size_t i = 0; i < cm.size(); ++i) cm[i] = make_int2(lat->chi_map[i].r, pack_perm(lat->chi_map[i].perm));
-        CK(f->chi_map.upload(cm.data(), cm.size(), st));
-        CK(f->chi_onsite.upload(lat->chi_onsite.data(), lat->chi_onsite.size(), st));
-        CK(f->chi_dr.upload(lat->chi_dr.data(), lat->chi_dr.size(), st));
+        tabs.add(f->chi_map, cm.data(), cm.size());
+        tabs.add(f->chi_onsite, lat->chi_onsite.data(), lat->chi_onsite.size());
+        tabs.add(f->chi_dr, lat->chi_dr.data(), lat->chi_dr.size());
         CK(f->chi.alloc(lat->chi_map.size() * g.nc * ts));
         if (g.nc != 16 && !f->ntan) {
             const chik::Displacements D = chik::merge(lat->chi_dr);
@@ -2120,6 +2150,7 @@ static sr_status flow_create(const sr_lattice* lat, int n_freq, const double* fr
             }
         }
     }
+    CK(tabs.upload(f->tables, st));
     // state
     CK(f->gam.alloc((size_t)g.N * ts));
     CK(f->G.alloc((size_t)g.nent * ts));
