@@ -6,8 +6,11 @@
 // of a 32-byte sector per corner; pairs related by symmetry repeat the same sum.  Here the frequency
 // pairs are split over the blocks, whose threads sum whole rows (all irreducible sites and
 // components, consecutive lanes), and the last block to finish adds the partial rows in a fixed
-// order and maps them onto the pairs.  (-w1, -w2) reads the same rows as (w1, w2), so half of the
-// frequency pairs are taken with doubled weight.  k_chi_k had one thread per momentum and a cosine per
+// order and maps them onto the pairs.  (-w1, -w2) reads the same corners as (w1, w2) with the sites
+// exchanged the same way, as s = w1 + w2 and u = w1 - w2 change their signs together, so half of the
+// frequency pairs are taken with doubled weight.  Where |w1| = |w2| one of the two is zero, which
+// counts as positive: the pair and its mirror image read one the plain, the other the exchanged entry,
+// and the value goes half to each.  k_chi_k had one thread per momentum and a cosine per
 // pair: the displacements are merged up to sign (the cosine is even) and a warp shares a momentum.
 // Square J1-J2 range 7, 48 frequencies, 64 x 64 momenta (one GB300): k_chi 149 -> 25 us (37
 // with a loop over the corners and one group of rows), k_chi_k 110 -> 23 us.  Latency bounds the sum (a chain of
@@ -63,6 +66,7 @@ k_chi_sum(Geo g, Tabs tb, const double* __restrict__ w, const double* __restrict
           double* __restrict__ Sd) {
     __shared__ double y[kMaxFreq + 1], yg[kMaxFreq + 1], Wn[kMaxFreq + 1];
     __shared__ Desc<double> dsc[kPass], dex[kPass];
+    __shared__ bool even[kPass];      // |w1| = |w2|
     __shared__ double on_sum[NC];
     __shared__ int last;
     extern __shared__ double acc[];   // [group][plain, exchanged][c * Ns + r]
@@ -82,7 +86,10 @@ k_chi_sum(Geo g, Tabs tb, const double* __restrict__ w, const double* __restrict
             const int i = tid < n ? tid : tid - n, idx = b0 + i, p = idx / (2 * K), q = idx - p * 2 * K, qk = q < K ? q : q - K;
             const double xp = y[p], xq = q < K ? y[qk] : -y[qk], W = 2.0 * Wn[p] * Wn[qk];
             Desc<double>& d = tid < n ? dsc[i] : dex[i];
-            if (tid < n) make_desc<double, true>(xp + xq, 0.0, xp - xq, 1, 0, tb, g, d, W);
+            if (tid < n) {
+                make_desc<double, true>(xp + xq, 0.0, xp - xq, 1, 0, tb, g, d, W);
+                even[i] = qk == p;
+            }
             else make_desc<double, true>(xp + xq, xq - xp, 0.0, 2, 0, tb, g, d, W);
             for (int k = d.n; k < 4; ++k) {   // always four corners: their loads need no loop
                 d.off[k] = d.off[0];
@@ -101,7 +108,9 @@ k_chi_sum(Geo g, Tabs tb, const double* __restrict__ w, const double* __restrict
                 double v = 0.0;
 #pragma unroll
                 for (int k = 0; k < 4; ++k) v = fma(wt[k], __ldg(G + d.off[k] + e), v);
-                if (d.swap) x += v; else a += v;
+                if (even[i]) { a = fma(0.5, v, a); x = fma(0.5, v, x); }
+                else if (d.swap) x += v;
+                else a += v;
             }
             acc[gi * 2 * row + e] += a;
             acc[(gi * 2 + 1) * row + e] += x;
