@@ -2614,8 +2614,8 @@ static sr_status adj_prepare_pair(sr_flow* f) {
     const Geo& g = f->g;
     if (!f->pk_on || f->prec != SR_FP64 || g.nc == 16) return SR_OK;
     const int Ns = g.Ns, nc = g.nc, row = Ns * nc, np = f->nprod, nst = f->pk.nst;
-    const size_t sm = nc == 2 ? pairk::adj_smem<2>(g.N, Ns, f->pk.rv, nst, np) : pairk::adj_smem<4>(g.N, Ns, f->pk.rv, nst, np);
-    if (sm > 227 * 1024 || f->pk.rv / 2 > 128) return SR_OK;
+    const size_t sm = nc == 2 ? pairk::adj_smem<2>(g.N, Ns, nst, np) : pairk::adj_smem<4>(g.N, Ns, nst, np);
+    if (sm > 227 * 1024 || Ns > 128) return SR_OK;
     // the fold needs the exchange to permute the stored entries
     std::vector<int> hit(row, 0);
     for (int r = 0; r < Ns; ++r)
@@ -2641,7 +2641,7 @@ static sr_status adj_prepare_pair(sr_flow* f) {
     for (int o = 0; o < row; ++o)   // h_goff runs over r * nc + c
         for (int k = f->h_goff[o]; k < f->h_goff[o + 1]; ++k) idx[fill[f->h_gidx[k]]++] = (o % nc) * Ns + o / nc;
     cudaStream_t st = f->stream;
-    if (f->Pbar.alloc(f->Pd.n) != cudaSuccess) {
+    if (f->Pbar.alloc((size_t)f->pk.nrow * nc * nst * (f->has_swap ? 2 : 1)) != cudaSuccess) {
         cudaGetLastError();
         f->Pbar.p = nullptr;
         return SR_OK;

@@ -2,16 +2,20 @@
 // after the shared device helpers).  Eq. frg:flowexplicit:2particle, one CTA per stored (s, u, t)
 // triple.
 //
-// s and u channels.  The projected products are those of commuting two-spin operators, so they are
-// diagonal in the common eigenbasis of sigma^c sigma^c: a row enters as its NC eigenvalues
-//     SU2  s: (d + s, d - 3 s)               u: (d - s, d + 3 s)
-//     XYZ  s: sum_c chi_e(c) Gamma^cc        u: Gamma^00 - sum_{c > 0} chi_e(c) Gamma^cc
-// (chi_e: the signs of sigma^c sigma^c on the four Bell states) and a node costs one multiply-add
-// per value instead of the 3 (SU2) or 4 (XYZ) of the component products.  Interpolation is linear,
-// so the eigenvalues are formed once per right-hand side (k_pair_pack) and interpolated themselves;
-// under the s <-> u relation, which flips the sign of the density, an s row reads minus the u row
-// and the other way round.  A thread interpolates the same values of both rows and multiplies them
-// in registers: no shared memory but the descriptors, no barrier between nodes.
+// s and u channels.  A thread interpolates both rows of a site and multiplies them in registers,
+// component by component: no shared memory but the descriptors, no barrier between nodes.  With
+// A, B the rows and a, b, c the three spin components in turn, the projected products are
+//     SU2  d: dA dB + 3 sA sB                    s: dA sB + sA dB -/+ 2 sA sB         (s / u channel)
+//     XYZ  0: sum_c Ac Bc                        a: A0 Ba + Aa B0 -/+ (Ab Bc + Ac Bb)
+// SU2 keeps sum dd, sum (ds + sd) and sum ss of each channel (four multiply-adds per node), XYZ the
+// four components.  (The products are diagonal in the common eigenbasis of sigma^c sigma^c, one
+// multiply-add per value; but a component is then a difference of eigenvalues, and one that is a
+// factor smaller than the others loses that factor in precision.  Whole right-hand side in that form
+// and in this one: square range 7 FP64 10.5 / 10.8 ms, pyrochlore range 6 FP32 8.2 / 8.4, Heisenberg-
+// Kitaev range 5 FP64 2.9 / 3.1.)
+// Their rows are stored site by site, so that a site's components come in one load; a row and its
+// s <-> u image, which flips the sign of the density, share the storage (a weight set each for the
+// density and the spin components).
 // t channel.  Interpolated component rows go to shared memory for the lattice sum: register tiles of
 // the dense contraction over pairs of sites (FP32; FP64 with many products) or a list of the
 // distinct products (FP64, whose pipe allows no padding); on-site terms in registers.
@@ -42,11 +46,10 @@ struct Tab {
     const double* mult; // FP64: multiplicity as a value
     const int2* prod;   // LIST: offsets (row A, row B) of every product
     int nprod;
-    int su_u;           // offset of the u rows of the packed state; the t rows follow at su_t
-    int su_t;
+    int su_t;           // offset of the t rows [component][site]; the s / u rows [site][component] start the packed state
     int on;             // on-site rows, each with its successor in t: [triple][2][component]
     int ex_su, ex_t;    // distance of the exchanged rows (0: the exchange is trivial)
-    int rv, nst;        // values of an s / u row, sites of a t row (both padded)
+    int rv, nst;        // stride of the s / u rows, sites of a t row (both padded)
     int nrow;           // stored triples
 };
 
@@ -56,10 +59,19 @@ constexpr int kSU = 128;   // s and u nodes whose descriptors share a pass
 constexpr int kT = 64;     // t nodes whose descriptors share a pass
 
 
+// Unit of an s / u row: the values a thread takes, whole sites and whole 16-byte chunks.
+template <typename R, int NC> __host__ __device__ constexpr int unit_values() { return vec<R>() > NC ? vec<R>() : NC; }
+template <typename R, int NC> __host__ __device__ constexpr int unit_sites() { return unit_values<R, NC>() / NC; }
+template <typename R, int NC> __host__ __device__ constexpr int units(int Ns) { return (Ns + unit_sites<R, NC>() - 1) / unit_sites<R, NC>(); }
+constexpr int kAcc = 4;    // partial sums of a site in the s and u channels
+
 // Descriptors in shared memory: arrays over the nodes of a pass (consecutive threads write
-// consecutive nodes) of corner offsets and corner weights, per row; t rows have a weight set for
-// the density and one for the spin components.
-template <typename R> __host__ __device__ constexpr size_t su_bytes() { return 2 * (16 + 4 * sizeof(R)) * kSU; }
+// consecutive nodes) of corner offsets and corner weights, per row, with a weight set for the density
+// and one for the spin components.  The s / u rows in FP64 have the latter alone and the density's
+// sign in bit 0 of the offset (offsets are even): its integer operations are free beside the FP64 pipe,
+// and the shared memory decides how many CTAs of a small lattice are resident.
+template <typename R> __host__ __device__ constexpr bool sign_in_offset() { return sizeof(R) == 8; }
+template <typename R> __host__ __device__ constexpr size_t su_bytes() { return 2 * (16 + (sign_in_offset<R>() ? 4 : 8) * sizeof(R)) * kSU; }
 template <typename R> __host__ __device__ constexpr size_t t_bytes() { return 2 * (16 + 8 * sizeof(R)) * kT; }
 
 __host__ __device__ inline size_t r16(size_t b) { return (b + 15) & ~size_t(15); }
@@ -67,11 +79,11 @@ __host__ __device__ inline size_t r16(size_t b) { return (b + 15) & ~size_t(15);
 // Shared memory of a triple: mesh, then a region for descriptors and rows, reused at the end for the
 // contraction's result and the threads' partial sums.
 template <typename R, int NC>
-__host__ __device__ inline size_t smem_bytes(int N, int rv, int nst, size_t nC, int threads) {
-    const int CH = rv / vec<R>(), NG = threads / CH, U = 2 * NC * nst / vec<R>(), S = threads / U;
+__host__ __device__ inline size_t smem_bytes(int N, int Ns, int nst, size_t nC, int threads) {
+    const int CH = units<R, NC>(Ns), NG = threads / CH, U = 2 * NC * nst / vec<R>(), S = threads / U;
     const size_t dsu = su_bytes<R>(), dt = t_bytes<R>() + sizeof(R) * 2 * NC * kT;
     const size_t work = r16(dt) + sizeof(R) * qrows<R>() * 2 * NC * nst;
-    const size_t fin = r16(sizeof(R) * nC) + r16(sizeof(R) * 2 * NG * rv) + r16(sizeof(R) * 2 * S * NC * nst);
+    const size_t fin = r16(sizeof(R) * nC) + r16(sizeof(R) * NG * kAcc * CH * unit_sites<R, NC>()) + r16(sizeof(R) * 2 * S * NC * nst);
     const size_t a = work > dsu ? work : dsu;
     return r16(sizeof(R) * 2 * N) + (a > fin ? a : fin);
 }
@@ -190,41 +202,60 @@ __device__ __forceinline__ void interp(const R* __restrict__ P, const int4 o, co
     for (int i = 0; i < V; ++i) v[i] = fmadd(w[3], c[3][i], fmadd(w[2], c[2][i], fmadd(w[1], c[1][i], w[0] * c[0][i])));
 }
 
-// Signs of sigma^c sigma^c on the Bell states: every product of two is minus the third, as
-// (sx sx)(sy sy) = -sz sz asks for.
-__host__ __device__ constexpr int bell(int e, int c) { return c == 0 ? 1 : (e == 3 ? -1 : (c - 1 == e ? -1 : 1)); }
-
-// Eigenvalue e of the components g[NC], s (SGN = 1) or u (SGN = -1) channel.
-template <int NC, typename T>
-__host__ __device__ __forceinline__ T eigen(const T* g, int e, int SGN) {
-    if (NC == 2) return SGN > 0 ? (e == 0 ? g[0] + g[1] : g[0] - 3 * g[1]) : (e == 0 ? g[0] - g[1] : g[0] + 3 * g[1]);
-    T a = g[0];
-#pragma unroll
-    for (int c = 1; c < NC; ++c) a += (SGN * bell(e, c) > 0) ? g[c] : -g[c];
-    return a;
+__device__ __forceinline__ float flip_sign(float x, int bit) { return __int_as_float(__float_as_int(x) ^ (bit << 31)); }
+__device__ __forceinline__ double flip_sign(double x, int bit) {
+    return __hiloint2double(__double2hiint(x) ^ (bit << 31), __double2loint(x));
 }
-// Component c of the operator with eigenvalues p[NC].
-template <int NC, typename T>
-__device__ __forceinline__ T component(const T* p, int c, int SGN) {
-    if (NC == 2) {
-        if (c == 0) return T(0.25) * (3 * p[0] + p[1]);
-        return SGN > 0 ? T(0.25) * (p[0] - p[1]) : T(0.25) * (p[1] - p[0]);
-    }
-    T a = p[0];
+
+// Interpolated unit of an s / u row; wt: weights of the spin components, wt + dens those of the density
+// (FP64: their signs in the offsets).
+template <typename R, int NC>
+__device__ __forceinline__ void interp_unit(const R* __restrict__ P, const int4 o, const R* wt, int dens, R* v) {
+    constexpr int VS = unit_values<R, NC>();
+    R ws[4], wd[4], c[4][VS];
+    const int of[4] = {o.x, o.y, o.z, o.w};
+    lds_w(wt, ws);
+    if constexpr (!sign_in_offset<R>()) lds_w(wt + dens, wd);
 #pragma unroll
-    for (int e = 1; e < NC; ++e) a += bell(e, c) > 0 ? p[e] : -p[e];
-    if (c > 0) {
-        a = bell(0, c) > 0 ? p[0] : -p[0];
-#pragma unroll
-        for (int e = 1; e < NC; ++e) a += bell(e, c) > 0 ? p[e] : -p[e];
-        if (SGN < 0) a = -a;
+    for (int k = 0; k < 4; ++k) {
+        if constexpr (sign_in_offset<R>()) wd[k] = flip_sign(ws[k], of[k]);
+        ld_n<VS>(P + (sign_in_offset<R>() ? of[k] & ~1 : of[k]), c[k]);
     }
-    return T(0.25) * a;
+#pragma unroll
+    for (int i = 0; i < VS; ++i) {
+        const R* w = i % NC == 0 ? wd : ws;
+        v[i] = fmadd(w[3], c[3][i], fmadd(w[2], c[2][i], fmadd(w[1], c[1][i], w[0] * c[0][i])));
+    }
+}
+
+// Partial sums of a site plus the product of its rows a, b: SU2 sum dd, sum (ds + sd), sum ss of the s
+// channel, sum ss of the u channel; XYZ the components.
+template <bool S_CH, int NC, typename R>
+__device__ __forceinline__ void su_products(const R* a, const R* b, R* acc) {
+    if constexpr (NC == 2) {
+        acc[0] = fmadd(a[0], b[0], acc[0]);
+        acc[1] = fmadd(a[0], b[1], fmadd(a[1], b[0], acc[1]));
+        acc[S_CH ? 2 : 3] = fmadd(a[1], b[1], acc[S_CH ? 2 : 3]);
+    } else {
+        acc[0] = fmadd(a[0], b[0], fmadd(a[1], b[1], fmadd(a[2], b[2], fmadd(a[3], b[3], acc[0]))));
+#pragma unroll
+        for (int c = 1; c < 4; ++c) {
+            const int e = c % 3 + 1, f = e % 3 + 1;
+            acc[c] = fmadd(a[0], b[c], fmadd(a[c], b[0], acc[c]));
+            acc[c] = fmadd(S_CH ? -a[e] : a[e], b[f], fmadd(S_CH ? -a[f] : a[f], b[e], acc[c]));
+        }
+    }
+}
+// Component c from a site's partial sums.
+template <int NC, typename R>
+__device__ __forceinline__ R su_component(const R* acc, int c) {
+    if constexpr (NC == 2) return c == 0 ? fmadd(R(3), acc[2] + acc[3], acc[0]) : fmadd(R(2), acc[3] - acc[2], acc[1]);
+    else return acc[c];
 }
 
 // One stored frequency triple, all sites and components, written to dG (FP64).
 // TILE: register tiles TM x TN of the dense contraction, NT per thread; LIST (TM = 1): NT products
-// per thread.  Needs blockDim.x >= rv / V and >= 2 NC nst / V.
+// per thread.  Needs blockDim.x >= units(Ns) and >= 2 NC nst / V.
 template <typename R, int NC, int TM, int TN, int NT>
 __device__ __forceinline__ void triple(const Geo& g, const Tabs& tb, const Tab& td, const R* __restrict__ P,
                                        const R* __restrict__ nx, const R* __restrict__ nW, const int* __restrict__ ncount,
@@ -250,13 +281,15 @@ __device__ __forceinline__ void triple(const Geo& g, const Tabs& tb, const Tab& 
     const R w1p = (s + t + u) * R(0.5), w2p = (s - t - u) * R(0.5), w1 = (s - t + u) * R(0.5), w2 = (s + t - u) * R(0.5);
 
     // ---- s and u channels
-    const int CH = rv / V, NG = nth / CH, my_g = tid / CH, my_c = tid - my_g * CH;
-    R ps[V], pu[V];
+    constexpr int VS = unit_values<R, NC>(), SPU = unit_sites<R, NC>();
+    const int CH = units<R, NC>(Ns), NG = nth / CH, my_g = tid / CH, my_c = tid - my_g * CH;
+    R psu[kAcc * SPU];
 #pragma unroll
-    for (int i = 0; i < V; ++i) ps[i] = pu[i] = R(0);
+    for (int i = 0; i < kAcc * SPU; ++i) psu[i] = R(0);
     {
         int4* offs = reinterpret_cast<int4*>(work);                     // [row][node]
-        R* wts = reinterpret_cast<R*>(work + 2 * 16 * kSU);             // [row][node][corner]
+        R* wts = reinterpret_cast<R*>(work + 2 * 16 * kSU);             // [spin, density][row][node][corner]
+        constexpr int kDens = 2 * 4 * kSU;
         const int cs = si, cu = 2 * N + ui, ns = ncount[cs], n_all = ns + ncount[cu];
         for (int n0 = 0; n0 < n_all; n0 += kSU) {
             const int nn = min(kSU, n_all - n0);
@@ -280,12 +313,14 @@ __device__ __forceinline__ void triple(const Geo& g, const Tabs& tb, const Tab& 
                     R wt[4];
                     bool neg[4];
                     corners<sizeof(R) == 4>(is_s ? 0 : 2, c0, c1, is_s ? si : ui, flip, N, rv, off, wt, neg);
-                    // s rows read the s table, minus the u table below the diagonal; u rows the other way round
+                    if constexpr (!sign_in_offset<R>()) {
+                        R wd[4];
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        off[k] += so + ((neg[k] == is_s) ? td.su_u : 0);
-                        wt[k] = neg[k] ? -wt[k] : wt[k];
+                        for (int k = 0; k < 4; ++k) wd[k] = neg[k] ? -wt[k] : wt[k];
+                        st_w(wts + kDens + 4 * (r * kSU + i), wd);
                     }
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) off[k] += so + (sign_in_offset<R>() && neg[k] ? 1 : 0);
                     offs[r * kSU + i] = make_int4(off[0], off[1], off[2], off[3]);
                     st_w(wts + 4 * (r * kSU + i), wt);
                 }
@@ -293,19 +328,19 @@ __device__ __forceinline__ void triple(const Geo& g, const Tabs& tb, const Tab& 
             __syncthreads();
             if (my_g < NG) {
                 // adjacent groups, in one warp, take adjacent nodes
-                const R* Pc = P + my_c * V;
+                const R* Pc = P + my_c * VS;
                 const int e = min(max(ns - n0, 0), nn);
-                auto channel = [&](int i0, int i1, R* out) {
+                auto channel = [&](auto is_s, int i0, int i1) {
                     for (int i = i0 + my_g; i < i1; i += NG) {
-                        R a[V], b[V];
-                        interp(Pc, offs[i], wts + 4 * i, a);
-                        interp(Pc, offs[kSU + i], wts + 4 * (kSU + i), b);
+                        R a[VS], b[VS];
+                        interp_unit<R, NC>(Pc, offs[i], wts + 4 * i, kDens, a);
+                        interp_unit<R, NC>(Pc, offs[kSU + i], wts + 4 * (kSU + i), kDens, b);
 #pragma unroll
-                        for (int j = 0; j < V; ++j) out[j] = fmadd(a[j], b[j], out[j]);
+                        for (int j = 0; j < SPU; ++j) su_products<decltype(is_s)::value, NC>(a + j * NC, b + j * NC, psu + j * kAcc);
                     }
                 };
-                channel(0, e, ps);
-                channel(e, nn, pu);
+                channel(std::true_type{}, 0, e);
+                channel(std::false_type{}, e, nn);
             }
         }
     }
@@ -459,8 +494,9 @@ __device__ __forceinline__ void triple(const Geo& g, const Tabs& tb, const Tab& 
     __syncthreads();
     const size_t nC = LIST ? (size_t)td.nprod : (size_t)td.nk * nst * nst;
     R* C = reinterpret_cast<R*>(work);
-    R* su = reinterpret_cast<R*>(work + r16(sizeof(R) * nC));                              // [group][s, u][rv]
-    R* tt = reinterpret_cast<R*>(work + r16(sizeof(R) * nC) + r16(sizeof(R) * 2 * NG * rv));   // [stream][row][rt]
+    const int nsu = kAcc * SPU * CH;
+    R* su = reinterpret_cast<R*>(work + r16(sizeof(R) * nC));                              // [group][site][kAcc]
+    R* tt = reinterpret_cast<R*>(work + r16(sizeof(R) * nC) + r16(sizeof(R) * NG * nsu));     // [stream][row][rt]
 #pragma unroll
     for (int j = 0; j < NT; ++j) {
         const int id = tid + j * nth;
@@ -476,42 +512,37 @@ __device__ __forceinline__ void triple(const Geo& g, const Tabs& tb, const Tab& 
         }
     }
     if (my_g < NG) {
-        st16(su + (2 * my_g) * rv + my_c * V, ps);
-        st16(su + (2 * my_g + 1) * rv + my_c * V, pu);
+#pragma unroll
+        for (int i = 0; i < kAcc * SPU; i += V) st16(su + my_g * nsu + my_c * kAcc * SPU + i, psu + i);
     }
     if (in_stream) st16(tt + (2 * stream + rw) * rt + ct * V, pt);
     __syncthreads();
     // FP64 and long rows: the sums over groups and streams first, a value each (into the slots of the
-    // first group and stream), instead of every output summing all eigenvalues it mixes (square range 7
-    // FP64 11.85 -> 11.70 ms, pyrochlore FP32 8.39 -> 8.18; the short FP32 rows lose 3 % by the barrier)
+    // first group and stream), instead of every output summing the values it mixes
     constexpr bool kStage = sizeof(R) == 8 || TM == 8;
     if constexpr (kStage) {
-        for (int v = tid; v < 2 * rv + rt; v += nth) {
-            if (v < 2 * rv) {
+        for (int v = tid; v < nsu + rt; v += nth) {
+            if (v < nsu) {
                 R a = su[v];
-                for (int k = 1; k < NG; ++k) a += su[2 * k * rv + v];
+                for (int k = 1; k < NG; ++k) a += su[k * nsu + v];
                 su[v] = a;
             } else {
-                R a = tt[v - 2 * rv];
-                for (int k = 1; k < 2 * S; ++k) a += tt[k * rt + v - 2 * rv];
-                tt[v - 2 * rv] = a;
+                R a = tt[v - nsu];
+                for (int k = 1; k < 2 * S; ++k) a += tt[k * rt + v - nsu];
+                tt[v - nsu] = a;
             }
         }
         __syncthreads();
     }
     for (int o = tid; o < NC * Ns; o += nth) {
         const int c = o / Ns, r = o - c * Ns;
-        R es[NC], eu[NC], a = tt[c * nst + r], l = R(0);
+        R x[kAcc], a = tt[c * nst + r], l = R(0);
 #pragma unroll
-        for (int e = 0; e < NC; ++e) {
-            es[e] = su[e * Ns + r];
-            eu[e] = su[rv + e * Ns + r];
-            if constexpr (!kStage)
-                for (int k = 1; k < NG; ++k) {
-                    es[e] += su[(2 * k) * rv + e * Ns + r];
-                    eu[e] += su[(2 * k + 1) * rv + e * Ns + r];
-                }
-        }
+        for (int e = 0; e < kAcc; ++e) x[e] = su[r * kAcc + e];
+        if constexpr (!kStage)
+            for (int k = 1; k < NG; ++k)
+#pragma unroll
+                for (int e = 0; e < kAcc; ++e) x[e] += su[k * nsu + r * kAcc + e];
         if constexpr (!kStage)
             for (int k = 1; k < 2 * S; ++k) a += tt[k * rt + c * nst + r];
         const int nt = td.n_terms[r];
@@ -523,7 +554,7 @@ __device__ __forceinline__ void triple(const Geo& g, const Tabs& tb, const Tab& 
             else m = (R)(code >> 20);
             l = fmadd(m, C[code & 0xfffff], l);
         }
-        a += component<NC, R>(es, c, 1) + component<NC, R>(eu, c, -1);
+        a += su_component<NC, R>(x, c);
         dG[((size_t)(p * N + ti) * NC + c) * Ns + r] = (double)a - 2.0 * (double)l;
     }
 }
@@ -536,46 +567,20 @@ k_gamma_rhs_pair(Geo g, Tabs tb, Tab td, const R* __restrict__ P, const R* __res
     triple<R, NC, TM, TN, NT>(g, tb, td, P, nx, nW, ncount, dG, p0 + (int)(blockIdx.x / g.N), blockIdx.x % g.N, smem);
 }
 
-// Eigenvalue e of components given as float pairs (hi + lo), rounded once: the sum of the FP64
-// components in FP32 arithmetic (two-term sums with their exact error, Knuth 1969).  FP64 additions and
-// conversions would bound the packing (36 per site for XYZ, 2 per clock and SM).
-template <int NC>
-__device__ __forceinline__ float eigen_pair(const float* hi, const float* lo, int e, int SGN) {
-    float h = hi[0], l = lo[0];
-    auto add = [&](float x, float xl) {
-        const float t = h + x, b = t - h;
-        l += (h - (t - b)) + (x - b) + xl;
-        h = t;
-    };
-    if (NC == 2) {
-        const bool pos = (SGN > 0) == (e == 0);
-        const float x = pos ? hi[1] : -hi[1], xl = pos ? lo[1] : -lo[1];
-        add(x, xl);
-        if (e == 1) add(2.0f * x, 2.0f * xl);
-    } else {
-#pragma unroll
-        for (int c = 1; c < NC; ++c) {
-            const bool pos = SGN * bell(e, c) > 0;
-            add(pos ? hi[c] : -hi[c], pos ? lo[c] : -lo[c]);
-        }
-    }
-    return h + l;
-}
-
-// Packed state: s and u eigenvalue rows and component rows of every stored triple, and the same of
-// the exchanged pairs when the site exchange is not trivial (the padding stays zero).  A block takes
-// whole rows, staged in shared memory (FP32: as float pairs), so that a component is read and
-// converted once; kPackThreads threads, grid-stride over the rows.
+// Packed state: s / u rows and t rows of every stored triple, and the same of the exchanged pairs when
+// the site exchange is not trivial (the padding stays zero).  A block takes whole rows, staged in
+// shared memory, so that a component is read and converted once; kPackThreads threads, grid-stride
+// over the rows.
 constexpr int kPackThreads = 256;
 template <typename R, int NC> __host__ __device__ constexpr size_t pack_smem(int Ns) {
-    return sizeof(double) * NC * (kPackThreads > Ns ? kPackThreads : Ns);
+    return sizeof(R) * NC * (kPackThreads > Ns ? kPackThreads : Ns);
 }
 
 template <typename R, int NC>
 __device__ __forceinline__ void pack_rows(const Geo& g, const Tabs& tb, const Tab& td, const double* __restrict__ G,
                                           R* __restrict__ P, unsigned char* smem) {
     const int Ns = g.Ns, RB = max(1, kPackThreads / Ns), cap = RB * Ns;   // rows of a block, their sites
-    R* sh = reinterpret_cast<R*>(smem);                                   // [component][site] (and the low parts)
+    R* sh = reinterpret_cast<R*>(smem);                                   // [component][site]
     const bool small = Ns <= kPackThreads;
     const int my_row = small ? (int)threadIdx.x / Ns : 0, first = small ? (int)threadIdx.x - my_row * Ns : (int)threadIdx.x;
     for (int row0 = blockIdx.x * RB; row0 < td.nrow; row0 += gridDim.x * RB) {
@@ -584,34 +589,24 @@ __device__ __forceinline__ void pack_rows(const Geo& g, const Tabs& tb, const Ta
         const double* src = G + (size_t)row * NC * Ns;
         for (int r = first; on && r < Ns; r += kPackThreads)
 #pragma unroll
-            for (int c = 0; c < NC; ++c) {
-                const double x = src[c * Ns + r];
-                const R h = (R)x;
-                sh[c * cap + my_row * Ns + r] = h;
-                if (sizeof(R) == 4) sh[(NC + c) * cap + my_row * Ns + r] = isfinite(h) ? (R)(x - (double)h) : R(0);
-            }
+            for (int c = 0; c < NC; ++c) sh[c * cap + my_row * Ns + r] = (R)src[c * Ns + r];
         __syncthreads();
         for (int r = first; on && r < Ns; r += kPackThreads)
             for (int x = 0; x < (td.ex_t ? 2 : 1); ++x) {
                 const int rs = my_row * Ns + (x ? tb.swap_r[r] : r), pm = x ? tb.swap_perm[r] : 0xe4;
-                R v[NC], lo[NC];
+                R v[NC];
 #pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    const int cs = perm_of(pm, c);
-                    v[c] = sh[cs * cap + rs];
-                    lo[c] = sizeof(R) == 4 ? sh[(NC + cs) * cap + rs] : R(0);
-                }
-                R* ps = P + (size_t)(x ? td.ex_su : 0) + (size_t)row * td.rv + r;
+                for (int c = 0; c < NC; ++c) v[c] = sh[perm_of(pm, c) * cap + rs];
+                R* ps = P + (size_t)(x ? td.ex_su : 0) + (size_t)row * td.rv + r * NC;
                 R* pt = P + td.su_t + (size_t)(x ? td.ex_t : 0) + (size_t)row * NC * td.nst + r;
+                if constexpr (NC * sizeof(R) >= 16) {
+#pragma unroll
+                    for (int c = 0; c < NC; c += vec<R>()) st16(ps + c, v + c);
+                } else {
+                    *reinterpret_cast<float2*>(ps) = make_float2(v[0], v[1]);
+                }
 #pragma unroll
                 for (int c = 0; c < NC; ++c) {
-                    if constexpr (sizeof(R) == 4) {
-                        ps[c * Ns] = eigen_pair<NC>(v, lo, c, 1);
-                        ps[td.su_u + c * Ns] = eigen_pair<NC>(v, lo, c, -1);
-                    } else {
-                        ps[c * Ns] = eigen<NC, R>(v, c, 1);
-                        ps[td.su_u + c * Ns] = eigen<NC, R>(v, c, -1);
-                    }
                     pt[c * td.nst] = v[c];
                     if (x == 0 && r == 0) {
                         R* o = P + td.on + (size_t)row * 2 * NC + c;
@@ -697,14 +692,17 @@ inline bool choose(const Variant* v, int count, int N, int Ns, int nc, int nk, i
     constexpr int V = vec<R>();
     for (int i = 0; i < count; ++i) {
         if (v[i].nc != nc) continue;
-        const int nst = (Ns + v[i].pad - 1) / v[i].pad * v[i].pad, rv = (nc * Ns + V - 1) / V * V;
+        const int nst = (Ns + v[i].pad - 1) / v[i].pad * v[i].pad;
+        // (FP64: the rows of both layouts have one stride, see pair_adj.cuh)
+        const int CH = nc == 2 ? units<R, 2>(Ns) : units<R, 4>(Ns);
+        const int rv = sizeof(R) == 8 ? nc * nst : CH * (nc == 2 ? unit_values<R, 2>() : unit_values<R, 4>());
         const bool list = v[i].tm == 1;
         const long T = list ? nprod : (long)nk * (nst / v[i].tm) * (nst / v[i].tn);
-        const long need = std::max(std::max((T + v[i].nt - 1) / v[i].nt, (long)rv / V), 2L * nc * nst / V);
+        const long need = std::max(std::max((T + v[i].nt - 1) / v[i].nt, (long)CH), 2L * nc * nst / V);
         const int th = (int)std::max(64L, (need + 31) / 32 * 32);
         if (th > v[i].max_threads) continue;
         const size_t nC = list ? (size_t)nprod : (size_t)nk * nst * nst;
-        const size_t sm = nc == 2 ? smem_bytes<R, 2>(N, rv, nst, nC, th) : smem_bytes<R, 4>(N, rv, nst, nC, th);
+        const size_t sm = nc == 2 ? smem_bytes<R, 2>(N, Ns, nst, nC, th) : smem_bytes<R, 4>(N, Ns, nst, nC, th);
         if (sm > 227 * 1024) continue;
         pl->variant = i;
         pl->threads = th;
@@ -736,14 +734,13 @@ inline bool build_tables(const sr_lattice* lat, int N, bool fp32, bool has_swap,
     if (!ok) return false;
     const Variant& v = fp32 ? kF32[pl->variant] : kF64[pl->variant];
     const long nrow = (long)N * (N + 1) / 2 * N, ex = has_swap ? 2 : 1;
-    pl->size = ex * nrow * (2L * td.rv + (long)nc * td.nst) + 2 * nc * nrow;
+    pl->size = ex * nrow * ((long)td.rv + (long)nc * td.nst) + 2 * nc * nrow;
     if (pl->size >= (1L << 31)) return false;   // 32-bit offsets
     td.nrow = (int)nrow;
     td.ex_su = has_swap ? (int)(nrow * td.rv) : 0;
     td.ex_t = has_swap ? (int)(nrow * nc * td.nst) : 0;
-    td.su_u = (int)(ex * nrow * td.rv);
-    td.su_t = (int)(2 * ex * nrow * td.rv);
-    td.on = (int)(ex * nrow * (2L * td.rv + (long)nc * td.nst));
+    td.su_t = (int)(ex * nrow * td.rv);
+    td.on = (int)(ex * nrow * ((long)td.rv + (long)nc * td.nst));
     if (v.tm == 1)
         for (const int2& p : prods)
             pl->prod.push_back(make_int2(p.x % nc * td.nst + p.x / nc, p.y % nc * td.nst + p.y / nc));

@@ -5,18 +5,20 @@
 // k_gamma_adj was bound by the FP64 pipe (86 % busy), most of it work beside the flow equations: the
 // products and their derivatives component by component, and compare-and-swap loops of double
 // additions in shared memory.  Here
-//   * s and u channels run in the eigenbasis of pair.cuh: with the output's adjoint o_e (a constant of
-//     the thread) the row adjoints are W o B and W o A, one product each;
+//   * s and u channels keep a site's components in the registers of one thread: with the output's
+//     adjoint o (constants of the thread) the row adjoints are W O(o) B and W O(o) A, O the symmetric
+//     matrix of the component products of pair.cuh, and the weight adjoint is A O(o) B;
 //   * the on-site factors' adjoints are summed once per node and component instead of by atomic
 //     additions from every site;
 //   * the adjoint of a node weight is summed from shared memory in a fixed order;
-//   * the transposed lookups add to accumulators in the packed layout (both eigenvalue tables, the
-//     component rows, and the same of the exchanged pairs), so lanes add to consecutive addresses;
-//     k_pair_fold maps them onto the state.
-// Heisenberg-Kitaev, range 5, 32 frequencies (one GB300): 15.8 -> 9.7 ms.  The FP64 pipe still bounds
-// it (81 % busy): 8 + 8 operations per value and node for the interpolation and its transpose, two per
-// product and node for the lattice sum.  Lists sorted by length (a warp runs as long as its longest):
-// 10.8 -> 9.9; registers capped for six CTAs instead of four: 9.9 -> 9.7.
+//   * the transposed lookups of all channels add to accumulators in the layout of the t rows (and the
+//     same of the exchanged pairs), so lanes add to consecutive addresses; k_pair_fold maps them onto
+//     the state.  (FP64 rows of both layouts have the same stride, so a packed offset serves both.)
+// Heisenberg-Kitaev, range 5, 32 frequencies (one GB300, a step's adjoint): 15.9 -> 9.4 ms, bound by the
+// FP64 pipe: 8 + 8 operations per value and node for the interpolation and its transpose, 2 x 16 per
+// site and node for the products, two per product and node for the lattice sum.  Lists sorted by length
+// (a warp runs as long as its longest): 10.9 -> 10.0 ms at that stage; registers capped for six CTAs
+// instead of four: 10.0 -> 9.8; one accumulator layout for all channels: 9.9 -> 9.4.
 #pragma once
 
 namespace pairk {
@@ -33,33 +35,48 @@ constexpr int kAN = 64;   // nodes whose descriptors share a pass
 constexpr int kAQ = 8;    // t-channel nodes per block of rows
 
 template <int NC>
-__host__ __device__ inline size_t adj_smem(int N, int Ns, int rv, int nst, int nprod) {
-    const int CH = rv / 2, rt = NC * nst;
-    const size_t su = (2 * 16 + 4 * 32 + 8) * (size_t)kAN + sizeof(double) * kAN * CH;
+__host__ __device__ inline size_t adj_smem(int N, int Ns, int nst, int nprod) {
+    const int CH = units<double, NC>(Ns), rt = NC * nst;
+    const size_t su = (2 * 16 + 2 * 32 + 8) * (size_t)kAN + sizeof(double) * kAN * CH;
     const size_t t = (4 * 48 + 8) * (size_t)kAN + sizeof(double) * (kAQ * 2 * rt + kAQ * 4 * NC + kAQ * 2 * NC * Ns);
     return r16(sizeof(double) * 2 * N) + r16(sizeof(double) * NC * Ns) + r16(sizeof(double) * nprod) + (su > t ? su : t) + 64;
 }
 
-// Adjoint of component(): eigenvalue adjoint e from the component adjoints f[NC].
-template <int NC>
-__device__ __forceinline__ double eigen_bar(const double* f, int e, int SGN) {
-    if (NC == 2) {
-        const double fs = (SGN > 0) == (e == 0) ? f[1] : -f[1];
-        return 0.25 * fma(e == 0 ? 3.0 : 1.0, f[0], fs);
-    }
-    double a = f[0];
+// t = O(f) v: derivative of f . product(a, v) with respect to a (and, O being symmetric, the same for
+// the other row) of the s (S_CH) or u channel.
+template <bool S_CH, int NC>
+__device__ __forceinline__ void product_adjoint(const double* f, const double* v, double* t) {
+    if constexpr (NC == 2) {
+        t[0] = fma(f[0], v[0], f[1] * v[1]);
+        t[1] = fma(f[1], v[0], fma(3.0, f[0], S_CH ? -2.0 * f[1] : 2.0 * f[1]) * v[1]);
+    } else {
+        t[0] = fma(f[0], v[0], fma(f[1], v[1], fma(f[2], v[2], f[3] * v[3])));
 #pragma unroll
-    for (int c = 1; c < NC; ++c) a += SGN * bell(e, c) > 0 ? f[c] : -f[c];
-    return 0.25 * a;
+        for (int c = 1; c < 4; ++c) {
+            const int e = c % 3 + 1, g = e % 3 + 1;
+            t[c] = fma(f[0], v[c], f[c] * v[0]);
+            t[c] = fma(S_CH ? -f[e] : f[e], v[g], fma(S_CH ? -f[g] : f[g], v[e], t[c]));
+        }
+    }
 }
 
-__device__ __forceinline__ void red2(double* p, double w, const double* v) {
-    if ((__double_as_longlong(w) & 0x7fffffffffffffffLL) == 0) return;   // w == 0 (uniform in a group)
-    atomicAdd(p, w * v[0]);
-    atomicAdd(p + 1, w * v[1]);
+// Transposed lookup of a unit: corner weights w (density signs in the offsets), values t, component
+// rows nst apart.
+template <int NC>
+__device__ __forceinline__ void red_unit(double* q, const int4 o, const double* wt, const double* t, int nst) {
+    double w[4];
+    lds_w(wt, w);
+    const int of[4] = {o.x, o.y, o.z, o.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if ((__double_as_longlong(w[k]) & 0x7fffffffffffffffLL) == 0) continue;   // w == 0 (uniform in a group)
+        double* p = q + (of[k] & ~1);
+#pragma unroll
+        for (int c = 0; c < NC; ++c) atomicAdd(p + c * nst, (c == 0 ? flip_sign(w[k], of[k]) : w[k]) * t[c]);
+    }
 }
 
-// Abar += (d dGamma / d Gamma)^T fbar in the packed layout, Wbar += d dGamma / d W . fbar; one CTA per
+// Abar += (d dGamma / d Gamma)^T fbar in the layout of the t rows, Wbar += d dGamma / d W . fbar; one CTA per
 // stored triple.
 template <int NC>
 __global__ void __launch_bounds__(128, 6)
@@ -91,34 +108,26 @@ k_gamma_adj_pair(Geo g, Tabs tb, Tab td, AdjTab at, const double* __restrict__ P
     const double s = wm[si], t = wm[ti], u = wm[ui];
     const double w1p = (s + t + u) * 0.5, w2p = (s - t - u) * 0.5, w1 = (s - t + u) * 0.5, w2 = (s + t - u) * 0.5;
 
-    // ---- s and u channels: thread (two values of a row, node group)
+    // ---- s and u channels: thread (site, node group)
     {
-        const int CH = rv / 2, NG = nth / CH, my_g = tid / CH, my_c = tid - my_g * CH;
+        const int CH = units<double, NC>(Ns), NG = nth / CH, my_g = tid / CH, my_c = tid - my_g * CH;
         int4* offs = reinterpret_cast<int4*>(work);                                 // [row][node]
-        double* wts = reinterpret_cast<double*>(work + 2 * 16 * kAN);               // [row][raw, times W][node][corner]
-        double* z = wts + 4 * 4 * kAN;                                              // [node][chunk]: o A B
-        for (int half = 0; half < 2; ++half) {
-            const bool is_s = half == 0;
+        double* wts = reinterpret_cast<double*>(work + 2 * 16 * kAN);               // [row][node][corner]
+        double* Wq = wts + 2 * 4 * kAN;                                             // [node]
+        double* z = Wq + kAN;                                                       // [node][site]: A O(o) B
+        double o[NC];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) o[c] = my_g < NG ? ob[c * Ns + my_c] : 0.0;
+        auto channel = [&](auto s_channel) {
+            constexpr bool is_s = decltype(s_channel)::value;
             const int cidx = is_s ? si : 2 * N + ui, nq = ncount[cidx];
-            double o[2] = {0.0, 0.0};
-            if (my_g < NG)
-#pragma unroll
-                for (int j = 0; j < 2; ++j) {
-                    const int v = 2 * my_c + j;
-                    if (v < row) {
-                        const int e = v / Ns, r = v - e * Ns;
-                        double f[NC];
-#pragma unroll
-                        for (int c = 0; c < NC; ++c) f[c] = ob[c * Ns + r];
-                        o[j] = eigen_bar<NC>(f, e, is_s ? 1 : -1);
-                    }
-                }
             for (int n0 = 0; n0 < nq; n0 += kAN) {
                 const int nn = min(kAN, nq - n0);
                 __syncthreads();
                 for (int idx = tid; idx < 2 * nn; idx += nth) {
                     const int r = idx >= nn ? 1 : 0, i = idx - r * nn;
-                    const double x = nx[(size_t)cidx * g.nmax + n0 + i], W = nW[(size_t)cidx * g.nmax + n0 + i];
+                    const double x = nx[(size_t)cidx * g.nmax + n0 + i];
+                    if (r == 0) Wq[i] = nW[(size_t)cidx * g.nmax + n0 + i];
                     const double y0 = r ? (is_s ? x - w1 : w1p + x) : (is_s ? w1p - x : w1 + x);
                     const double y1 = r ? (is_s ? x - w2 : w2 - x) : x - w2p;
                     const double m0 = mag(y0), m1 = mag(y1);
@@ -127,39 +136,34 @@ k_gamma_adj_pair(Geo g, Tabs tb, Tab td, AdjTab at, const double* __restrict__ P
                     const int so = swap ? td.ex_su : 0;
                     const bool flip = is_s ? less(s, m1) : less(m0, u);
                     int off[4];
-                    double wt[4], ww[4];
+                    double wt[4];
                     bool neg[4];
                     corners<false>(is_s ? 0 : 2, c0, c1, is_s ? si : ui, flip, N, rv, off, wt, neg);
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        off[k] += so + ((neg[k] == is_s) ? td.su_u : 0);
-                        wt[k] = neg[k] ? -wt[k] : wt[k];
-                        ww[k] = W * wt[k];
-                    }
+                    for (int k = 0; k < 4; ++k) off[k] += so + (neg[k] ? 1 : 0);
                     offs[r * kAN + i] = make_int4(off[0], off[1], off[2], off[3]);
-                    st_w(wts + 4 * ((2 * r) * kAN + i), wt);
-                    st_w(wts + 4 * ((2 * r + 1) * kAN + i), ww);
+                    st_w(wts + 4 * (r * kAN + i), wt);
                 }
                 __syncthreads();
                 if (my_g < NG)
                     for (int i = my_g; i < nn; i += NG) {
-                        double a[2], b[2], w[4];
+                        double a[NC], b[NC], ta[NC], tb_[NC];
                         const int4 oa = offs[i], obb = offs[kAN + i];
-                        interp(P + 2 * my_c, oa, wts + 4 * i, a);
-                        interp(P + 2 * my_c, obb, wts + 4 * (2 * kAN + i), b);
-                        const double tb_[2] = {o[0] * b[0], o[1] * b[1]}, ta_[2] = {o[0] * a[0], o[1] * a[1]};
-                        z[i * CH + my_c] = fma(a[1], tb_[1], a[0] * tb_[0]);
-                        double* q = Pbar + 2 * my_c;
-                        lds_w(wts + 4 * (kAN + i), w);
-                        red2(q + oa.x, w[0], tb_);
-                        red2(q + oa.y, w[1], tb_);
-                        red2(q + oa.z, w[2], tb_);
-                        red2(q + oa.w, w[3], tb_);
-                        lds_w(wts + 4 * (3 * kAN + i), w);
-                        red2(q + obb.x, w[0], ta_);
-                        red2(q + obb.y, w[1], ta_);
-                        red2(q + obb.z, w[2], ta_);
-                        red2(q + obb.w, w[3], ta_);
+                        interp_unit<double, NC>(P + NC * my_c, oa, wts + 4 * i, 0, a);
+                        interp_unit<double, NC>(P + NC * my_c, obb, wts + 4 * (kAN + i), 0, b);
+                        product_adjoint<is_s, NC>(o, b, ta);
+                        product_adjoint<is_s, NC>(o, a, tb_);
+                        const double W = Wq[i];
+                        double zz = 0.0;
+#pragma unroll
+                        for (int c = 0; c < NC; ++c) {
+                            zz = fma(a[c], ta[c], zz);
+                            ta[c] *= W;
+                            tb_[c] *= W;
+                        }
+                        z[i * CH + my_c] = zz;
+                        red_unit<NC>(Pbar + my_c, oa, wts + 4 * i, ta, nst);
+                        red_unit<NC>(Pbar + my_c, obb, wts + 4 * (kAN + i), tb_, nst);
                     }
                 __syncthreads();
                 for (int i = tid; i < nn; i += nth) {
@@ -168,7 +172,9 @@ k_gamma_adj_pair(Geo g, Tabs tb, Tab td, AdjTab at, const double* __restrict__ P
                     atomicAdd(&Wbar[(size_t)cidx * g.nmax + n0 + i], a);
                 }
             }
-        }
+        };
+        channel(std::true_type{});
+        channel(std::false_type{});
     }
     __syncthreads();
 
@@ -180,7 +186,6 @@ k_gamma_adj_pair(Geo g, Tabs tb, Tab td, AdjTab at, const double* __restrict__ P
     double* fac = rows + kAQ * 2 * rt;                                            // [q][C, D][factor, adjoint][component]
     double* z = fac + kAQ * 4 * NC;                                               // [q][2 row]
     const double* Pt = P + td.su_t;
-    double* Pbt = Pbar + td.su_t;
     const int cidx = N + ti, nq = ncount[cidx];
     for (int n0 = 0; n0 < nq; n0 += kAN) {
         const int nn = min(kAN, nq - n0);
@@ -281,7 +286,7 @@ k_gamma_adj_pair(Geo g, Tabs tb, Tab td, AdjTab at, const double* __restrict__ P
                         const int4 of = offs[rw * kAN + q0 + q];
                         double w[4];
                         lds_w(wts + 4 * (rw * kAN + q0 + q), w);
-                        double* b = Pbt + c * nst + r;
+                        double* b = Pbar + c * nst + r;
                         const int o4[4] = {of.x, of.y, of.z, of.w};
 #pragma unroll
                         for (int k = 0; k < 4; ++k)
@@ -304,7 +309,7 @@ k_gamma_adj_pair(Geo g, Tabs tb, Tab td, AdjTab at, const double* __restrict__ P
                 const int o4[4] = {of.x, of.y, of.z, of.w};
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
-                    if (w[k] != 0.0) atomicAdd(Pbt + o4[k] + c * nst, (c > 0 ? mag(w[k]) : w[k]) * a);
+                    if (w[k] != 0.0) atomicAdd(Pbar + o4[k] + c * nst, (c > 0 ? mag(w[k]) : w[k]) * a);
             }
             // weight adjoints: 16 lanes per node, fixed order
             for (int base = tid >> 4; base < qn; base += nth >> 4) {
@@ -318,8 +323,8 @@ k_gamma_adj_pair(Geo g, Tabs tb, Tab td, AdjTab at, const double* __restrict__ P
     }
 }
 
-// Gammabar from the packed accumulators: transpose of pack_site, a block per stored triple (shared
-// memory: NC * Ns doubles).
+// Gammabar from the accumulators: transpose of the exchange in pack_rows, a block per stored triple
+// (shared memory: NC * Ns doubles).
 template <int NC>
 __global__ void k_pair_fold(Geo g, Tabs tb, Tab td, const double* __restrict__ Pbar, double* __restrict__ Gbar) {
     extern __shared__ double acc[];
@@ -327,27 +332,14 @@ __global__ void k_pair_fold(Geo g, Tabs tb, Tab td, const double* __restrict__ P
     for (int row = blockIdx.x; row < td.nrow; row += gridDim.x) {
         for (int x = 0; x < (td.ex_t ? 2 : 1); ++x) {
             for (int r = threadIdx.x; r < Ns; r += blockDim.x) {
-                const double* bs = Pbar + (x ? td.ex_su : 0) + (size_t)row * td.rv + r;
-                const double* bt = Pbar + td.su_t + (x ? td.ex_t : 0) + (size_t)row * NC * td.nst + r;
-                double sb[NC], ub[NC], v[NC];
-#pragma unroll
-                for (int e = 0; e < NC; ++e) { sb[e] = bs[e * Ns]; ub[e] = bs[td.su_u + e * Ns]; }
-#pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    double a = bt[c * td.nst];
-                    if (NC == 2)
-                        a += c == 0 ? (sb[0] + sb[1]) + (ub[0] + ub[1]) : (sb[0] - ub[0]) + 3.0 * (ub[1] - sb[1]);
-                    else
-#pragma unroll
-                        for (int e = 0; e < NC; ++e) a += c == 0 ? sb[e] + ub[e] : (bell(e, c) > 0 ? sb[e] - ub[e] : ub[e] - sb[e]);
-                    v[c] = a;
-                }
+                const double* bt = Pbar + (x ? td.ex_t : 0) + (size_t)row * NC * td.nst + r;
                 // (the exchange permutes the stored entries: no two threads meet)
                 const int rs = x ? tb.swap_r[r] : r, pm = x ? tb.swap_perm[r] : 0xe4;
 #pragma unroll
                 for (int c = 0; c < NC; ++c) {
                     double& a = acc[perm_of(pm, c) * Ns + rs];
-                    a = x ? a + v[c] : v[c];
+                    const double v = bt[c * td.nst];
+                    a = x ? a + v : v;
                 }
             }
             __syncthreads();
