@@ -224,6 +224,17 @@ sr_status sr_flow_destroy(sr_flow* flow);
 sr_status sr_flow_set_tensor_cores(sr_flow* flow, int on);
 sr_status sr_flow_tensor_cores(const sr_flow* flow, int* on);
 
+/* Whether the vertex flow runs on a packed copy of the state (on, the default where the lattice has
+ * such a kernel and the copy found memory when the flow was created) or on the stored state.  Off
+ * frees the copy and with it the packed adjoint: for SU2 / XYZ two values per entry (four with a
+ * non-trivial site exchange), FP64 or FP32 as the precision, and half of that for the adjoint; for TRI
+ * one or two FP32 / FP64 values per entry.  Slower: 1.3 to 8 times.  FP32-mixed flows then hold an
+ * FP32 copy of the entries instead.  Synchronises.  Errors: SR_EUNSUPPORTED (on, and the lattice has
+ * no packed kernel), SR_ENOMEM (the flow stays as it was), SR_EINVAL (null, or the flow is in a
+ * batch). */
+sr_status sr_flow_set_packed(sr_flow* flow, int on);
+sr_status sr_flow_packed(const sr_flow* flow, int* on);
+
 /* ---- tangent-linear flow: derivatives of the flow along coupling directions ---- */
 
 /* Like sr_flow_init (FP64), but the state carries, with every value, its derivatives along
@@ -295,7 +306,7 @@ sr_status sr_flow_initial_vertex_adjoint(sr_flow* flow, int n_par, const double*
 typedef struct sr_batch sr_batch;
 
 /* Group flows (all SR_FP32_MIXED, on the current device; the batch keeps pointers to them,
- * so they must outlive it).  The vertex flow of every instance runs in one persistent kernel
+ * so they must outlive it).  Flows on the packed and on the stored state may be mixed.  The vertex flow of every instance runs in one persistent kernel
  * whose CTAs take (instance, stored triple) units from an atomic counter, largest instances
  * first; the paper's analogue is its dynamically balanced work units (Sec. 4.4).  TRI flows
  * (16 basis functions) run their own vertex kernel inside the batch's step; their self-energy

@@ -78,6 +78,8 @@ def load_library():
             "sr_flow_tangents": [vp, ip],
             "sr_flow_set_tensor_cores": [vp, i],
             "sr_flow_tensor_cores": [vp, ip],
+            "sr_flow_set_packed": [vp, i],
+            "sr_flow_packed": [vp, ip],
             "sr_measure_susceptibility_tangent": [vp, i, dp, dp, dp],
             "sr_flow_sizes": [vp, lp, ip, ip],
             "sr_flow_rhs": [vp, d, vp, vp],
@@ -334,6 +336,17 @@ class Flow:
     @tensor_cores.setter
     def tensor_cores(self, on: bool):
         _check(self._lib.sr_flow_set_tensor_cores(self.h, 1 if on else 0))
+
+    @property
+    def packed(self) -> bool:
+        """Whether the vertex flow runs on a packed copy of the state (False frees it)."""
+        v = C.c_int()
+        _check(self._lib.sr_flow_packed(self.h, C.byref(v)))
+        return bool(v.value)
+
+    @packed.setter
+    def packed(self, on: bool):
+        _check(self._lib.sr_flow_set_packed(self.h, 1 if on else 0))
 
     def set_step_limit(self, n: int):
         _check(self._lib.sr_flow_set_step_limit(self.h, int(n)))

@@ -1525,7 +1525,8 @@ struct sr_flow {
     DevBuf<int4> tlat_items;
     int tlat_n_items = 0;
     // SU2 / XYZ vertex flow (pairk::): tables, kernel variant and packed state
-    bool pk_on = false;
+    bool pk_on = false, pk_plan = false;   // the packed state serves the flow; it has a plan
+    size_t n_packed = 0;                   // values of the packed state (either core)
     pairk::Tab pk{};
     int pk_variant = -1, pk_threads = 0;
     size_t pk_smem = 0;
@@ -1535,11 +1536,12 @@ struct sr_flow {
     trid::Tab td{};
     trid::Choice<float> tdf;
     trid::Choice<double> tdd;
-    bool td_on = false, td_graded = false;
+    bool td_on = false, td_plan = false, td_graded = false;
     DevBuf<unsigned char> td_tables;
     int* td_flag = nullptr;
     DevBuf<float> Pf;
     DevBuf<double> Pd;
+    std::shared_ptr<int> in_use = std::make_shared<int>(0);   // shared with the batches that hold its pointers
 
     Tabs tabs() const {
         Tabs t;
@@ -1596,6 +1598,30 @@ static sr_status prof_end(sr_flow* f, int id, cudaEvent_t b) {
     CK(cudaEventRecord(e, f->stream));
     f->ev[id].push_back({b, e});
     return SR_OK;
+}
+
+// FP32 copy of the state that the kernels on the stored state read.
+static cudaError_t alloc_copy(sr_flow* f) {
+    if (f->prec != SR_FP32_MIXED || f->Gf.p) return cudaSuccess;
+    const cudaError_t e = f->Gf.alloc(f->g.nc == 16 ? (size_t)f->g.nent : (size_t)f->g.nentp * (f->has_swap ? 2 : 1));
+    if (e != cudaSuccess) f->Gf.alloc(0);
+    return e;
+}
+
+// The packed state of a flow that has a plan for it (its padding stays zero).
+static cudaError_t packed_alloc(sr_flow* f) {
+    cudaError_t e = f->prec == SR_FP64 ? f->Pd.alloc(f->n_packed) : f->Pf.alloc(f->n_packed);
+    if (e == cudaSuccess && f->pk_plan)
+        e = f->prec == SR_FP64 ? cudaMemsetAsync(f->Pd.p, 0, sizeof(double) * f->n_packed, f->stream)
+                               : cudaMemsetAsync(f->Pf.p, 0, sizeof(float) * f->n_packed, f->stream);
+    if (e != cudaSuccess) {
+        f->Pd.alloc(0);
+        f->Pf.alloc(0);
+        return e;
+    }
+    f->pk_on = f->pk_plan;
+    f->td_on = f->td_plan;
+    return e;
 }
 
 // SU2 / XYZ: pack the state G_s for the vertex kernel.
@@ -1771,6 +1797,18 @@ static sr_status refresh_shadow(sr_flow* f, const double* G_s, float* Gf_s) {
     return SR_OK;
 }
 
+// Frees the packed state (and the adjoint that reads it): the kernels on the stored state take over.
+static sr_status packed_release(sr_flow* f) {
+    f->pk_on = f->td_on = false;
+    f->Pd.alloc(0);
+    f->Pf.alloc(0);
+    if (f->pka_on) {
+        f->pka_on = f->adj_ready = false;
+        f->Pbar.alloc(0);
+    }
+    return refresh_shadow(f, f->G.p, f->Gf.p);
+}
+
 // ----------------------------------------------------------------------------- ABI: lattice
 
 extern "C" sr_status sr_lattice_create(const sr_lattice_desc* desc, sr_lattice** out) {
@@ -1875,7 +1913,6 @@ static sr_status flow_create(const sr_lattice* lat, int n_freq, const double* fr
     f->ntan = npar > 0 ? kTan : 0;
     f->ts = 1 + f->ntan;
     const int ts = f->ts;
-    size_t n_packed = 0;   // values of the packed state
     TableSet tabs;
     std::vector<double> init_host = lat->init_gamma;
     if (npar > 0) {
@@ -1960,7 +1997,7 @@ static sr_status flow_create(const sr_lattice* lat, int n_freq, const double* fr
         tabs.add(f->dgath_idx, dg.data(), dg.size());
         pairk::Plan pl;
         if (!f->ntan && pairk::build_plan(lat, n_freq, precision != SR_FP64, f->has_swap, prods, goff, gidx, &pl)) {
-            f->pk_on = true;
+            f->pk_plan = true;
             f->pk = pl.td;
             f->pk_variant = pl.variant;
             f->pk_threads = pl.threads;
@@ -1975,7 +2012,7 @@ static sr_status flow_create(const sr_lattice* lat, int n_freq, const double* fr
             f->pk.prod = (const int2*)(base + o_prod);
             f->pk.kap = (const int*)(base + o_kap);
             f->pk.mult = (const double*)(base + o_mult);
-            n_packed = (size_t)pl.size;
+            f->n_packed = (size_t)pl.size;
             CK(ensure_smem(precision == SR_FP64 ? (const void*)pairk::kernel_f64(pl.variant) : (const void*)pairk::kernel_f32(pl.variant),
                            pl.smem));
         }
@@ -2127,7 +2164,7 @@ static sr_status flow_create(const sr_lattice* lat, int n_freq, const double* fr
                 if (on) CK(ensure_smem((const void*)f->tdf.fn, f->tdf.smem));
             }
             if (on) {
-                f->td_on = true;
+                f->td_plan = true;
                 f->td_graded = pl.graded;
                 TableBlob tbl;
                 const size_t o_pack = tbl.add(pl.pack), o_fmap = tbl.add(pl.fmap), o_ent = tbl.add(pl.ent), o_runs = tbl.add(pl.runs),
@@ -2146,7 +2183,7 @@ static sr_status flow_create(const sr_lattice* lat, int n_freq, const double* fr
                 td.nrow = (int)nrow;
                 const unsigned long long half = (unsigned long long)(pl.graded ? Ns : 2 * Ns);
                 td.div_half = half > 1 ? (unsigned)((0x100000000ULL + half - 1) / half) : 0u;
-                n_packed = (size_t)g.nent * (pl.graded ? 1 : 2);
+                f->n_packed = (size_t)g.nent * (pl.graded ? 1 : 2);
             }
         }
     }
@@ -2156,21 +2193,12 @@ static sr_status flow_create(const sr_lattice* lat, int n_freq, const double* fr
     CK(f->G.alloc((size_t)g.nent * ts));
     CK(f->dgam.alloc((size_t)g.N * ts));
     CK(f->dG.alloc((size_t)g.nent * ts));
-    if (n_packed > 0) {   // where it finds no memory the kernels on the stored state serve the flow
-        const cudaError_t e = precision == SR_FP64 ? f->Pd.alloc(n_packed) : f->Pf.alloc(n_packed);
-        if (e == cudaErrorMemoryAllocation) {
-            cudaGetLastError();
-            f->Pd.p = nullptr;
-            f->Pf.p = nullptr;
-            f->pk_on = f->td_on = false;
-        } else {
-            CK(e);
-            if (f->Pd.p && f->pk_on) CK(cudaMemsetAsync(f->Pd.p, 0, sizeof(double) * n_packed, st));   // padding stays zero
-            if (f->Pf.p && f->pk_on) CK(cudaMemsetAsync(f->Pf.p, 0, sizeof(float) * n_packed, st));
-        }
+    if (f->n_packed > 0) {   // where it finds no memory the kernels on the stored state serve the flow
+        const cudaError_t e = packed_alloc(f.get());
+        if (e == cudaErrorMemoryAllocation) cudaGetLastError();
+        else CK(e);
     }
-    if (precision == SR_FP32_MIXED && !(f->td_on && !f->td_graded) && !f->pk_on)
-        CK(f->Gf.alloc(g.nc == 16 ? (size_t)g.nent : (size_t)g.nentp * (f->has_swap ? 2 : 1)));
+    if (!(f->td_on && !f->td_graded) && !f->pk_on) CK(alloc_copy(f.get()));
     CK(f->nx.alloc((size_t)3 * g.N * g.nmax));
     CK(f->nW.alloc((size_t)3 * g.N * g.nmax * ts));
     CK(f->nWf.alloc((size_t)3 * g.N * g.nmax));
@@ -2251,12 +2279,9 @@ extern "C" sr_status sr_flow_set_tensor_cores(sr_flow* f, int on) {
     if (!f) return fail(SR_EINVAL, "null flow");
     if (on && !(f->prec == SR_FP32_MIXED && tc_supported(f->g.nc, f->g.nsp, f->dense)))
         return fail(SR_EUNSUPPORTED, "tensor-core lattice sum needs an FP32-mixed SU2 flow with at most 64 padded sites");
-    if (on && !f->Gf.p) {   // its copy of the state (a flow on the packed state has none)
-        if (f->Gf.alloc((size_t)f->g.nentp * (f->has_swap ? 2 : 1)) != cudaSuccess) {
-            cudaGetLastError();
-            f->Gf.p = nullptr;
-            return fail(SR_ENOMEM, "no device memory for the tensor-core path's copy of the state");
-        }
+    if (on && alloc_copy(f) != cudaSuccess) {   // (a flow on the packed state has none)
+        cudaGetLastError();
+        return fail(SR_ENOMEM, "no device memory for the tensor-core path's copy of the state");
     }
     f->use_tc = on != 0;
     return SR_OK;
@@ -2265,6 +2290,33 @@ extern "C" sr_status sr_flow_set_tensor_cores(sr_flow* f, int on) {
 extern "C" sr_status sr_flow_tensor_cores(const sr_flow* f, int* on) {
     if (!f || !on) return fail(SR_EINVAL, "null argument");
     *on = f->use_tc ? 1 : 0;
+    return SR_OK;
+}
+
+extern "C" sr_status sr_flow_set_packed(sr_flow* f, int on) {
+    if (!f) return fail(SR_EINVAL, "null flow");
+    if ((on != 0) == (f->pk_on || f->td_on)) return SR_OK;
+    if (on && f->n_packed == 0) return fail(SR_EUNSUPPORTED, "no packed-state kernel for this flow");
+    if (f->in_use.use_count() > 1) return fail(SR_EINVAL, "the flow is in a batch, which holds its buffers");
+    CK(cudaStreamSynchronize(f->stream));
+    if (on) {
+        if (packed_alloc(f) != cudaSuccess) {
+            cudaGetLastError();
+            return fail(SR_ENOMEM, "no device memory for the packed state (%zu values)", f->n_packed);
+        }
+        f->adj_ready = f->pka_on;   // the next adjoint takes the packed form again
+        return SR_OK;
+    }
+    if (alloc_copy(f) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(SR_ENOMEM, "no device memory for the FP32 copy of the state");
+    }
+    return packed_release(f);
+}
+
+extern "C" sr_status sr_flow_packed(const sr_flow* f, int* on) {
+    if (!f || !on) return fail(SR_EINVAL, "null argument");
+    *on = f->pk_on || f->td_on ? 1 : 0;
     return SR_OK;
 }
 
@@ -2920,7 +2972,7 @@ struct BInst {
     int* ncount;
     long unit0;     // first work unit (stored triple) of this instance
     int qc;         // integration nodes per shared-memory block
-    int kind;       // 0 SU2 / XYZ on the packed state (pairk), 2 XYZ general kernel, 3 TRI
+    int kind;       // 0 SU2 / XYZ on the packed state (pairk), 1 SU2 and 2 XYZ on the stored state, 3 TRI
     int with_swap;
     pairk::Tab pk;  // kind 0: tables and packed state
     float* P;
@@ -3048,11 +3100,12 @@ static PersistentPair persistent_pair(int variant) {
     return nullptr;
 }
 
-// Persistent kernel of an instance kind (0: packed-state kernel in the given variant, 2: XYZ general
-// kernel; TRI instances, kind 3, always run their own kernels); every size class holds instances of
-// one kind and variant.
+// Persistent kernel of an instance kind (0: packed-state kernel in the given variant, 1, 2: SU2 and XYZ
+// kernels on the stored state; TRI instances, kind 3, always run their own kernels); every size class
+// holds instances of one kind and variant.
 static const void* persistent_fn(int kind, int variant) {
-    return kind == 0 ? (const void*)persistent_pair(variant) : (const void*)k_gamma_persistent<4, false>;
+    if (kind == 0) return (const void*)persistent_pair(variant);
+    return kind == 1 ? (const void*)k_gamma_persistent<2, true> : (const void*)k_gamma_persistent<4, false>;
 }
 
 // Euler update of every instance (y <- y - (Lambda_k - Lambda_k+1) f) and its FP32 shadow.
@@ -3155,6 +3208,7 @@ struct sr_batch {
     int force = 0;                    // 0: the autotuner picks the launch form per class,
                                       // 1: persistent kernels, 2: per-instance kernels
     std::vector<size_t> inst_smem;    // per instance: dynamic shared memory of its own kernel
+    std::vector<std::shared_ptr<int>> in_use;   // the flows' marks: their buffers stay where they are
     ~sr_batch() {
         for (cudaStream_t s : side) cudaStreamDestroy(s);
         for (cudaEvent_t e : join) cudaEventDestroy(e);
@@ -3174,6 +3228,8 @@ static void launch_class(sr_batch* b, int k, cudaStream_t st) {
             if (c.kind == 0) launch_gamma_pair(B.flow, B.dG, 0, B.g.npair, st);
             else if (c.kind == 3)
                 launch_gamma_tri(B.flow, B.G, B.Gf, B.dG, 0, B.g.npair, st);
+            else if (c.kind == 1)
+                k_gamma_rhs_f32<2, true><<<blocks, kThreads, sm, st>>>(B.g, B.tb, B.Gf, B.Gs, B.nxf, B.nWf, B.ncount, B.dG, 0);
             else
                 k_gamma_rhs_f32<4, false><<<blocks, kThreads, sm, st>>>(B.g, B.tb, B.Gf, B.Gs, B.nxf, B.nWf, B.ncount, B.dG, 0);
         }
@@ -3183,6 +3239,8 @@ static void launch_class(sr_batch* b, int k, cudaStream_t st) {
     unsigned long long* ctr = b->counter.p + k;
     if (c.kind == 0)
         persistent_pair(c.variant)<<<grid, c.threads, c.smem, st>>>(b->dinst.p, c.i_begin, c.i_end, c.u_begin, c.u_end, ctr, kUnitChunk);
+    else if (c.kind == 1)
+        k_gamma_persistent<2, true><<<grid, kThreads, c.smem, st>>>(b->dinst.p, c.i_begin, c.i_end, c.u_begin, c.u_end, ctr);
     else
         k_gamma_persistent<4, false><<<grid, kThreads, c.smem, st>>>(b->dinst.p, c.i_begin, c.i_end, c.u_begin, c.u_end, ctr);
 }
@@ -3384,6 +3442,7 @@ extern "C" sr_status sr_batch_create(int n, sr_flow* const* flows, sr_batch** ou
         if (!f) return fail(SR_EINVAL, "null flow %d", i);
         if (f->prec != SR_FP32_MIXED) return fail(SR_EUNSUPPORTED, "batched flows use the FP32-mixed kernels (flow %d is FP64)", i);
         b->flows.push_back(f);
+        b->in_use.push_back(f->in_use);
     }
     // instances grouped by kind and by the shared memory their vertex flow needs (each class
     // gets a persistent launch sized for it), largest first; within a class, largest instance
@@ -3392,9 +3451,7 @@ extern "C" sr_status sr_batch_create(int n, sr_flow* const* flows, sr_batch** ou
     std::vector<int> kind(n);
     for (int i = 0; i < n; ++i) {
         sr_flow* f = flows[i];
-        kind[i] = f->g.nc == 16 ? 3 : (f->pk_on ? 0 : 2);
-        if (kind[i] == 2 && f->g.nc == 2)
-            return fail(SR_EUNSUPPORTED, "flow %d: lattice too large for the batched SU2 kernel", i);
+        kind[i] = f->g.nc == 16 ? 3 : (f->pk_on ? 0 : (f->g.nc == 2 ? 1 : 2));
         if (kind[i] == 0) sm[i] = f->pk_smem;
         else if (kind[i] == 3) sm[i] = f->smem_rhs;
         else sm[i] = f32_smem_bytes(f->g.Ns, f->g.nsp, f->g.nc, f->nprod, f->dense);
