@@ -37,7 +37,8 @@
 
 namespace pairk {
 
-// Tables of one lattice and flow (device pointers, offsets in elements of the packed state).
+// Tables of one lattice and flow (device pointers).  The rows of a kind are addressed in chunks of 16
+// bytes, so that 31 bits reach every mesh and lattice whose state's entries 31 bits count.
 struct Tab {
     int nk;             // component pairs (row A, row B) of the lattice sum
     const int* kap;     // nk: cA | cB << 4
@@ -46,9 +47,9 @@ struct Tab {
     const double* mult; // FP64: multiplicity as a value
     const int2* prod;   // LIST: offsets (row A, row B) of every product
     int nprod;
-    int su_t;           // offset of the t rows [component][site]; the s / u rows [site][component] start the packed state
-    int on;             // on-site rows, each with its successor in t: [triple][2][component]
-    int ex_su, ex_t;    // distance of the exchanged rows (0: the exchange is trivial)
+    long su_t;          // offset of the t rows [component][site]; the s / u rows [site][component] start the packed state
+    long on;            // on-site rows, each with its successor in t: [triple][2][component]
+    int ex_su, ex_t;    // distance of the exchanged rows in 16-byte chunks (0: the exchange is trivial)
     int rv, nst;        // stride of the s / u rows, sites of a t row (both padded)
     int nrow;           // stored triples
 };
@@ -68,8 +69,8 @@ constexpr int kAcc = 4;    // partial sums of a site in the s and u channels
 // Descriptors in shared memory: arrays over the nodes of a pass (consecutive threads write
 // consecutive nodes) of corner offsets and corner weights, per row, with a weight set for the density
 // and one for the spin components.  The s / u rows in FP64 have the latter alone and the density's
-// sign in bit 0 of the offset (offsets are even): its integer operations are free beside the FP64 pipe,
-// and the shared memory decides how many CTAs of a small lattice are resident.
+// sign in bit 31 of the offset: its integer operations are free beside the FP64 pipe, and the shared
+// memory decides how many CTAs of a small lattice are resident.
 template <typename R> __host__ __device__ constexpr bool sign_in_offset() { return sizeof(R) == 8; }
 template <typename R> __host__ __device__ constexpr size_t su_bytes() { return 2 * (16 + (sign_in_offset<R>() ? 4 : 8) * sizeof(R)) * kSU; }
 template <typename R> __host__ __device__ constexpr size_t t_bytes() { return 2 * (16 + 8 * sizeof(R)) * kT; }
@@ -130,7 +131,7 @@ __device__ __forceinline__ bool less(double a, double b) { return __double_as_lo
 // Four corners of a row: cells a, b along the two free axes, the third index exact.  EA: the exact
 // axis (0 s, 1 t, 2 u); a, b are (t, u), (s, u) or (s, t).  flip: |s| < |u|.  Corner (i_s, j_t, k_u) is
 // stored at the pair (max, min) of i_s, k_u; below the diagonal (and on it for a flipped lookup) the
-// s <-> u relation flips the density's sign.
+// s <-> u relation flips the density's sign.  row: stride of a row in chunks.
 // SLOTS (FP32, bound by the L1 path): a corner goes to the slot of its index parities.  Consecutive
 // nodes share about half of their corners; in its slot a shared corner is read by the same load
 // instruction for the adjacent nodes that a warp handles, as one access to its lines.
@@ -194,17 +195,19 @@ __device__ __forceinline__ void interp(const R* __restrict__ P, const int4 o, co
     constexpr int V = vec<R>();
     R w[4], c[4][V];
     lds_w(wt, w);
-    ld16(P + o.x, c[0]);
-    ld16(P + o.y, c[1]);
-    ld16(P + o.z, c[2]);
-    ld16(P + o.w, c[3]);
+    ld16(P + (long)o.x * V, c[0]);
+    ld16(P + (long)o.y * V, c[1]);
+    ld16(P + (long)o.z * V, c[2]);
+    ld16(P + (long)o.w * V, c[3]);
 #pragma unroll
     for (int i = 0; i < V; ++i) v[i] = fmadd(w[3], c[3][i], fmadd(w[2], c[2][i], fmadd(w[1], c[1][i], w[0] * c[0][i])));
 }
 
-__device__ __forceinline__ float flip_sign(float x, int bit) { return __int_as_float(__float_as_int(x) ^ (bit << 31)); }
-__device__ __forceinline__ double flip_sign(double x, int bit) {
-    return __hiloint2double(__double2hiint(x) ^ (bit << 31), __double2loint(x));
+// x with its sign changed where bit 31 of o is set
+constexpr int kNeg = (int)0x80000000;
+__device__ __forceinline__ float flip_sign(float x, int o) { return __int_as_float(__float_as_int(x) ^ (o & kNeg)); }
+__device__ __forceinline__ double flip_sign(double x, int o) {
+    return __hiloint2double(__double2hiint(x) ^ (o & kNeg), __double2loint(x));
 }
 
 // Interpolated unit of an s / u row; wt: weights of the spin components, wt + dens those of the density
@@ -219,7 +222,7 @@ __device__ __forceinline__ void interp_unit(const R* __restrict__ P, const int4 
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         if constexpr (sign_in_offset<R>()) wd[k] = flip_sign(ws[k], of[k]);
-        ld_n<VS>(P + (sign_in_offset<R>() ? of[k] & ~1 : of[k]), c[k]);
+        ld_n<VS>(P + (long)(sign_in_offset<R>() ? of[k] & ~kNeg : of[k]) * vec<R>(), c[k]);
     }
 #pragma unroll
     for (int i = 0; i < VS; ++i) {
@@ -263,7 +266,7 @@ __device__ __forceinline__ void triple(const Geo& g, const Tabs& tb, const Tab& 
     constexpr int V = vec<R>(), QB = qrows<R>();
     constexpr bool LIST = TM == 1;
     const int tid = threadIdx.x, nth = blockDim.x, N = g.N, Ns = g.Ns;
-    const int rv = td.rv, nst = td.nst, rt = NC * nst;
+    const int nst = td.nst, rt = NC * nst;
     R* wm = reinterpret_cast<R*>(smem);
     R* ih = wm + N;
     unsigned char* work = smem + r16(sizeof(R) * 2 * N);
@@ -312,7 +315,7 @@ __device__ __forceinline__ void triple(const Geo& g, const Tabs& tb, const Tab& 
                     int off[4];
                     R wt[4];
                     bool neg[4];
-                    corners<sizeof(R) == 4>(is_s ? 0 : 2, c0, c1, is_s ? si : ui, flip, N, rv, off, wt, neg);
+                    corners<sizeof(R) == 4>(is_s ? 0 : 2, c0, c1, is_s ? si : ui, flip, N, td.rv / V, off, wt, neg);
                     if constexpr (!sign_in_offset<R>()) {
                         R wd[4];
 #pragma unroll
@@ -320,7 +323,7 @@ __device__ __forceinline__ void triple(const Geo& g, const Tabs& tb, const Tab& 
                         st_w(wts + kDens + 4 * (r * kSU + i), wd);
                     }
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) off[k] += so + (sign_in_offset<R>() && neg[k] ? 1 : 0);
+                    for (int k = 0; k < 4; ++k) off[k] += so + (sign_in_offset<R>() && neg[k] ? kNeg : 0);
                     offs[r * kSU + i] = make_int4(off[0], off[1], off[2], off[3]);
                     st_w(wts + 4 * (r * kSU + i), wt);
                 }
@@ -410,7 +413,7 @@ __device__ __forceinline__ void triple(const Geo& g, const Tabs& tb, const Tab& 
                     int off[4];
                     R wt[4], wd[4];
                     bool neg[4];
-                    corners<sizeof(R) == 4>(1, cw, c1, ti, less(m0, m1), N, rt, off, wt, neg);
+                    corners<sizeof(R) == 4>(1, cw, c1, ti, less(m0, m1), N, rt / V, off, wt, neg);
 #pragma unroll
                     for (int k = 0; k < 4; ++k) wd[k] = neg[k] ? -wt[k] : wt[k];
                     offs[r * kT + i] = make_int4(off[0] + so, off[1] + so, off[2] + so, off[3] + so);
@@ -597,8 +600,8 @@ __device__ __forceinline__ void pack_rows(const Geo& g, const Tabs& tb, const Ta
                 R v[NC];
 #pragma unroll
                 for (int c = 0; c < NC; ++c) v[c] = sh[perm_of(pm, c) * cap + rs];
-                R* ps = P + (size_t)(x ? td.ex_su : 0) + (size_t)row * td.rv + r * NC;
-                R* pt = P + td.su_t + (size_t)(x ? td.ex_t : 0) + (size_t)row * NC * td.nst + r;
+                R* ps = P + (size_t)(x ? td.ex_su : 0) * vec<R>() + (size_t)row * td.rv + r * NC;
+                R* pt = P + td.su_t + (size_t)(x ? td.ex_t : 0) * vec<R>() + (size_t)row * NC * td.nst + r;
                 if constexpr (NC * sizeof(R) >= 16) {
 #pragma unroll
                     for (int c = 0; c < NC; c += vec<R>()) st16(ps + c, v + c);
@@ -679,7 +682,7 @@ inline Kernel<double> kernel_f64(int id) {
 struct Plan {
     int variant = -1, threads = 0;
     size_t smem = 0;
-    long size = 0;   // elements of the packed state
+    long size = 0;   // values of the packed state
     Tab td{};
     std::vector<int> terms, n_terms, kap;
     std::vector<int2> prod;
@@ -734,13 +737,14 @@ inline bool build_tables(const sr_lattice* lat, int N, bool fp32, bool has_swap,
     if (!ok) return false;
     const Variant& v = fp32 ? kF32[pl->variant] : kF64[pl->variant];
     const long nrow = (long)N * (N + 1) / 2 * N, ex = has_swap ? 2 : 1;
-    pl->size = ex * nrow * ((long)td.rv + (long)nc * td.nst) + 2 * nc * nrow;
-    if (pl->size >= (1L << 31)) return false;   // 32-bit offsets
+    const long V = fp32 ? vec<float>() : vec<double>(), rt = (long)nc * td.nst;
+    if (ex * nrow * std::max((long)td.rv, rt) / V >= (1L << 31)) return false;   // 31-bit chunk offsets
+    pl->size = ex * nrow * (td.rv + rt) + 2 * nc * nrow;
     td.nrow = (int)nrow;
-    td.ex_su = has_swap ? (int)(nrow * td.rv) : 0;
-    td.ex_t = has_swap ? (int)(nrow * nc * td.nst) : 0;
-    td.su_t = (int)(ex * nrow * td.rv);
-    td.on = (int)(ex * nrow * ((long)td.rv + (long)nc * td.nst));
+    td.ex_su = has_swap ? (int)(nrow * td.rv / V) : 0;
+    td.ex_t = has_swap ? (int)(nrow * rt / V) : 0;
+    td.su_t = ex * nrow * td.rv;
+    td.on = ex * nrow * (td.rv + rt);
     if (v.tm == 1)
         for (const int2& p : prods)
             pl->prod.push_back(make_int2(p.x % nc * td.nst + p.x / nc, p.y % nc * td.nst + p.y / nc));

@@ -70,7 +70,7 @@ __device__ __forceinline__ void red_unit(double* q, const int4 o, const double* 
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         if ((__double_as_longlong(w[k]) & 0x7fffffffffffffffLL) == 0) continue;   // w == 0 (uniform in a group)
-        double* p = q + (of[k] & ~1);
+        double* p = q + (long)(of[k] & ~kNeg) * 2;
 #pragma unroll
         for (int c = 0; c < NC; ++c) atomicAdd(p + c * nst, (c == 0 ? flip_sign(w[k], of[k]) : w[k]) * t[c]);
     }
@@ -84,7 +84,7 @@ k_gamma_adj_pair(Geo g, Tabs tb, Tab td, AdjTab at, const double* __restrict__ P
                  const double* __restrict__ nW, const int* __restrict__ ncount, const double* __restrict__ fbar,
                  double* __restrict__ Pbar, double* __restrict__ Wbar) {
     extern __shared__ __align__(16) unsigned char smem[];
-    const int tid = threadIdx.x, nth = blockDim.x, N = g.N, Ns = g.Ns, rv = td.rv, nst = td.nst, rt = NC * nst;
+    const int tid = threadIdx.x, nth = blockDim.x, N = g.N, Ns = g.Ns, rc = td.rv / 2, nst = td.nst, rt = NC * nst;
     const int row = NC * Ns;
     double* wm = reinterpret_cast<double*>(smem);
     double* ih = wm + N;
@@ -138,9 +138,9 @@ k_gamma_adj_pair(Geo g, Tabs tb, Tab td, AdjTab at, const double* __restrict__ P
                     int off[4];
                     double wt[4];
                     bool neg[4];
-                    corners<false>(is_s ? 0 : 2, c0, c1, is_s ? si : ui, flip, N, rv, off, wt, neg);
+                    corners<false>(is_s ? 0 : 2, c0, c1, is_s ? si : ui, flip, N, rc, off, wt, neg);
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) off[k] += so + (neg[k] ? 1 : 0);
+                    for (int k = 0; k < 4; ++k) off[k] += so + (neg[k] ? kNeg : 0);
                     offs[r * kAN + i] = make_int4(off[0], off[1], off[2], off[3]);
                     st_w(wts + 4 * (r * kAN + i), wt);
                 }
@@ -202,7 +202,7 @@ k_gamma_adj_pair(Geo g, Tabs tb, Tab td, AdjTab at, const double* __restrict__ P
                 int off[4];
                 double wt[4];
                 bool neg[4];
-                corners<false>(h ? 2 : 1, c0, c1, ti, h ? less(m0, t) : less(m0, m1), N, rt, off, wt, neg);
+                corners<false>(h ? 2 : 1, c0, c1, ti, h ? less(m0, t) : less(m0, m1), N, rc, off, wt, neg);
                 const int slot = h ? 3 - r : r, add = h ? 0 : so;
 #pragma unroll
                 for (int k = 0; k < 4; ++k) wt[k] = neg[k] ? -wt[k] : wt[k];
@@ -226,8 +226,8 @@ k_gamma_adj_pair(Geo g, Tabs tb, Tab td, AdjTab at, const double* __restrict__ P
                 if (c > 0)
 #pragma unroll
                     for (int k = 0; k < 4; ++k) w[k] = mag(w[k]);
-                const double* b = Pt + at_;
-                const double val = fma(w[3], __ldg(b + of.w), fma(w[2], __ldg(b + of.z), fma(w[1], __ldg(b + of.y), w[0] * __ldg(b + of.x))));
+                auto at = [&](int o) { return __ldg(Pt + at_ + (long)o * 2); };
+                const double val = fma(w[3], at(of.w), fma(w[2], at(of.z), fma(w[1], at(of.y), w[0] * at(of.x))));
                 if (on) fac[(q * 4 + 2 * rw + 1) * NC + c] = val;   // raw row, replaced by its adjoint below
                 else rows[(q * 2 + rw) * rt + at_] = val;
             }
@@ -290,7 +290,7 @@ k_gamma_adj_pair(Geo g, Tabs tb, Tab td, AdjTab at, const double* __restrict__ P
                         const int o4[4] = {of.x, of.y, of.z, of.w};
 #pragma unroll
                         for (int k = 0; k < 4; ++k)
-                            if ((__double_as_longlong(w[k]) & 0x7fffffffffffffffLL) != 0) atomicAdd(b + o4[k], (c > 0 ? mag(w[k]) : w[k]) * vb);
+                            if ((__double_as_longlong(w[k]) & 0x7fffffffffffffffLL) != 0) atomicAdd(b + (long)o4[k] * 2, (c > 0 ? mag(w[k]) : w[k]) * vb);
                     }
             }
             __syncthreads();
@@ -309,7 +309,7 @@ k_gamma_adj_pair(Geo g, Tabs tb, Tab td, AdjTab at, const double* __restrict__ P
                 const int o4[4] = {of.x, of.y, of.z, of.w};
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
-                    if (w[k] != 0.0) atomicAdd(Pbar + o4[k] + c * nst, (c > 0 ? mag(w[k]) : w[k]) * a);
+                    if (w[k] != 0.0) atomicAdd(Pbar + (long)o4[k] * 2 + c * nst, (c > 0 ? mag(w[k]) : w[k]) * a);
             }
             // weight adjoints: 16 lanes per node, fixed order
             for (int base = tid >> 4; base < qn; base += nth >> 4) {
@@ -332,7 +332,7 @@ __global__ void k_pair_fold(Geo g, Tabs tb, Tab td, const double* __restrict__ P
     for (int row = blockIdx.x; row < td.nrow; row += gridDim.x) {
         for (int x = 0; x < (td.ex_t ? 2 : 1); ++x) {
             for (int r = threadIdx.x; r < Ns; r += blockDim.x) {
-                const double* bt = Pbar + (x ? td.ex_t : 0) + (size_t)row * NC * td.nst + r;
+                const double* bt = Pbar + (x ? (size_t)td.ex_t * 2 : 0) + (size_t)row * NC * td.nst + r;
                 // (the exchange permutes the stored entries: no two threads meet)
                 const int rs = x ? tb.swap_r[r] : r, pm = x ? tb.swap_perm[r] : 0xe4;
 #pragma unroll

@@ -110,3 +110,31 @@ def test_batch_takes_flows_on_the_stored_state(mode, autotune):
     flows[2].packed = False
     for f in single + flows:
         f.close()
+
+
+def test_mesh_beyond_31_bits_of_packed_values():
+    """The largest meshes keep the packed form: its offsets count chunks of four values."""
+    import torch
+
+    import paper_2109_13317_gb300 as sr
+    N, lam = 256, 0.7
+    lat = sr.Lattice.from_model(MODELS["kagome"](), 7)
+    mesh = sr.sr_frequency_mesh_exponential(N, 0.05, 20.0)
+    fl = sr.Flow(lat, mesh, lam, sr.SR_FP32_MIXED)
+    sr.Batch([fl]).close()
+    assert 2 * 2 * (2 * lat.N_s) * N * fl.npair >= 2 ** 31
+    assert fl.packed
+    gen = torch.Generator(device="cuda").manual_seed(4)
+    G = torch.randn(fl.n_gamma, dtype=torch.float64, device="cuda", generator=gen)
+    G.view(fl.shape())[[i * (i + 3) // 2 for i in range(N)], :, 0] = 0.0    # no density at s = u
+    fl.set_state(lam, torch.tensor(0.2 * np.tanh(mesh), device="cuda"), G)
+    out = []
+    for packed in (True, False):
+        fl.packed = packed
+        ds = torch.empty(N, dtype=torch.float64, device="cuda")
+        fl.rhs_pairs(lam, fl.npair - 2, fl.npair, ds, G)    # (the flow has its own copy of the state)
+        out.append(G.view(fl.shape())[-2:].clone())
+    # as test_gpu_pair.py: rounding of 6e-8 per product, at most linearly over ~1e3 terms of an output
+    for c in range(2):
+        assert _rel(out[0][:, :, c], out[1][:, :, c]) <= 1e-4
+    fl.close()
