@@ -1401,9 +1401,12 @@ struct DevBuf {
         if (p && !view) cudaFree(p);
         p = nullptr;
         view = false;
-        n = count;
+        n = 0;
         if (count == 0) return cudaSuccess;
-        return cudaMalloc((void**)&p, sizeof(T) * count);
+        const cudaError_t e = cudaMalloc((void**)&p, sizeof(T) * count);
+        if (e == cudaSuccess) n = count;
+        else p = nullptr;
+        return e;
     }
     cudaError_t upload(const T* host, size_t count, cudaStream_t st) {
         cudaError_t e = alloc(count);
@@ -1603,9 +1606,7 @@ static sr_status prof_end(sr_flow* f, int id, cudaEvent_t b) {
 // FP32 copy of the state that the kernels on the stored state read.
 static cudaError_t alloc_copy(sr_flow* f) {
     if (f->prec != SR_FP32_MIXED || f->Gf.p) return cudaSuccess;
-    const cudaError_t e = f->Gf.alloc(f->g.nc == 16 ? (size_t)f->g.nent : (size_t)f->g.nentp * (f->has_swap ? 2 : 1));
-    if (e != cudaSuccess) f->Gf.alloc(0);
-    return e;
+    return f->Gf.alloc(f->g.nc == 16 ? (size_t)f->g.nent : (size_t)f->g.nentp * (f->has_swap ? 2 : 1));
 }
 
 // The packed state of a flow that has a plan for it (its padding stays zero).
@@ -1693,6 +1694,8 @@ static void launch_gamma_tri(sr_flow* f, const double* G_s, const float* Gf_s, d
 // Right-hand side at cutoff lam for the state (gam_s, G_s [, Gf_s]) into (dgam_o, dG_o).
 static sr_status run_rhs(sr_flow* f, double lam, const double* gam_s, const double* G_s, const float* Gf_s,
                          double* dgam_o, double* dG_o, int pb = 0, int pe = -1) {
+    if (f->prec == SR_FP32_MIXED && !f->pk_on && !f->td_on && !Gf_s)
+        return fail(SR_ENOMEM, "no device memory for the FP32 copy of the state");
     const Geo& g = f->g;
     Tabs tb = f->tabs();
     cudaEvent_t e0 = nullptr;
@@ -1783,6 +1786,7 @@ static sr_status run_rhs(sr_flow* f, double lam, const double* gam_s, const doub
 
 static sr_status refresh_shadow(sr_flow* f, const double* G_s, float* Gf_s) {
     if (f->prec != SR_FP32_MIXED) return SR_OK;
+    if (!f->pk_on && !f->td_on && !f->Gf.p) return fail(SR_ENOMEM, "no device memory for the FP32 copy of the state");
     if (f->g.nc == 16) {
         if (f->td_on) return SR_OK;   // packed with the vertex launch
         const long n = f->g.nent;
@@ -1807,6 +1811,34 @@ static sr_status packed_release(sr_flow* f) {
         f->Pbar.alloc(0);
     }
     return refresh_shadow(f, f->G.p, f->Gf.p);
+}
+
+// An allocation step that found no memory, once more without the packed state, which the flow can do
+// without; with it again where that does not help.
+template <typename Alloc>
+static sr_status with_room(sr_flow* f, Alloc alloc) {
+    sr_status s = alloc();
+    if (s == SR_OK || cudaPeekAtLastError() != cudaErrorMemoryAllocation) return s;
+    cudaGetLastError();
+    if (!(f->pk_on || f->td_on) || f->in_use.use_count() > 1) return s;
+    CK(cudaStreamSynchronize(f->stream));
+    const bool had_copy = f->Gf.p != nullptr;
+    f->Pd.alloc(0);   // (what it held may be what the FP32 copy needs)
+    f->Pf.alloc(0);
+    if (alloc_copy(f) == cudaSuccess) {
+        if (sr_status e = packed_release(f)) return e;
+        if ((s = alloc()) == SR_OK) return s;
+    }
+    cudaGetLastError();
+    if (!had_copy) f->Gf.alloc(0);
+    if (packed_alloc(f) != cudaSuccess) {
+        cudaGetLastError();
+        f->pk_on = f->td_on = false;
+        alloc_copy(f);
+        cudaGetLastError();
+        refresh_shadow(f, f->G.p, f->Gf.p);
+    }
+    return s;
 }
 
 // ----------------------------------------------------------------------------- ABI: lattice
@@ -2279,7 +2311,7 @@ extern "C" sr_status sr_flow_set_tensor_cores(sr_flow* f, int on) {
     if (!f) return fail(SR_EINVAL, "null flow");
     if (on && !(f->prec == SR_FP32_MIXED && tc_supported(f->g.nc, f->g.nsp, f->dense)))
         return fail(SR_EUNSUPPORTED, "tensor-core lattice sum needs an FP32-mixed SU2 flow with at most 64 padded sites");
-    if (on && alloc_copy(f) != cudaSuccess) {   // (a flow on the packed state has none)
+    if (on && with_room(f, [&] { return alloc_copy(f) == cudaSuccess ? SR_OK : SR_ENOMEM; }) != SR_OK) {   // (a flow on the packed state has none)
         cudaGetLastError();
         return fail(SR_ENOMEM, "no device memory for the tensor-core path's copy of the state");
     }
@@ -2401,14 +2433,24 @@ extern "C" sr_status sr_flow_advance(sr_flow* f, double lambda_next, const doubl
 }
 
 static sr_status ensure_rk(sr_flow* f) {
-    if (f->y0G.p) return SR_OK;
+    if (f->kG[6].p) return SR_OK;
     const Geo& g = f->g;
-    CK(f->y0g.alloc(g.N));
-    CK(f->y0G.alloc(g.nent));
-    CK(f->stg.alloc(g.N));
-    CK(f->stG.alloc(g.nent));
-    for (int i = 0; i < 7; ++i) { CK(f->kg[i].alloc(g.N)); CK(f->kG[i].alloc(g.nent)); }
-    return SR_OK;
+    auto alloc = [&]() -> sr_status {
+        CK(f->y0g.alloc(g.N));
+        CK(f->y0G.alloc(g.nent));
+        CK(f->stg.alloc(g.N));
+        CK(f->stG.alloc(g.nent));
+        for (int i = 0; i < 7; ++i) { CK(f->kg[i].alloc(g.N)); CK(f->kG[i].alloc(g.nent)); }
+        return SR_OK;
+    };
+    return with_room(f, [&] {
+        const sr_status s = alloc();
+        if (s != SR_OK) {   // all of it or none
+            for (DevBuf<double>* b : {&f->y0G, &f->stG}) b->alloc(0);
+            for (DevBuf<double>& b : f->kG) b.alloc(0);
+        }
+        return s;
+    });
 }
 
 // One Dormand-Prince 5(4) step of size h from the current state; writes the fifth-order
@@ -2715,8 +2757,7 @@ static sr_status adj_prepare_pair(sr_flow* f) {
     return SR_OK;
 }
 
-static sr_status adj_prepare(sr_flow* f) {
-    if (f->adj_ready) return SR_OK;
+static sr_status adj_prepare_once(sr_flow* f) {
     const Geo& g = f->g;
     if (g.nc == 16) {
         // TRI: the vertex adjoint walks the forward lattice-sum table itself
@@ -2770,6 +2811,10 @@ static sr_status adj_prepare(sr_flow* f) {
     CK(cudaStreamSynchronize(st));
     f->adj_ready = true;
     return SR_OK;
+}
+
+static sr_status adj_prepare(sr_flow* f) {
+    return f->adj_ready ? SR_OK : with_room(f, [&] { return adj_prepare_once(f); });
 }
 
 static sr_status adj_check(const sr_flow* f) {
@@ -3452,6 +3497,7 @@ extern "C" sr_status sr_batch_create(int n, sr_flow* const* flows, sr_batch** ou
     for (int i = 0; i < n; ++i) {
         sr_flow* f = flows[i];
         kind[i] = f->g.nc == 16 ? 3 : (f->pk_on ? 0 : (f->g.nc == 2 ? 1 : 2));
+        if (!f->pk_on && !f->td_on && !f->Gf.p) return fail(SR_ENOMEM, "flow %d: no device memory for the FP32 copy of the state", i);
         if (kind[i] == 0) sm[i] = f->pk_smem;
         else if (kind[i] == 3) sm[i] = f->smem_rhs;
         else sm[i] = f32_smem_bytes(f->g.Ns, f->g.nsp, f->g.nc, f->nprod, f->dense);

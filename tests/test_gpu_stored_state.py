@@ -138,3 +138,53 @@ def test_mesh_beyond_31_bits_of_packed_values():
     for c in range(2):
         assert _rel(out[0][:, :, c], out[1][:, :, c]) <= 1e-4
     fl.close()
+
+
+@pytest.mark.parametrize("mixed", [False, True])
+def test_workspace_takes_the_room_of_the_packed_state(mixed):
+    """A Dormand-Prince workspace that finds no memory beside the packed state takes its room; one that
+    does not fit either way fails and leaves the flow as it was."""
+    import gc
+
+    import torch
+
+    import paper_2109_13317_gb300 as sr
+    mib = 1 << 20
+    lat = sr.Lattice.from_model(MODELS["kagome"](), 7)
+    mesh = sr.sr_frequency_mesh_exponential(64, 0.05, 20.0)
+    prec = sr.SR_FP32_MIXED if mixed else sr.SR_FP64
+    ref = sr.Flow(lat, mesh, 3.0, prec)
+    ref.step(2.5, sr.SR_RK_FIXED)
+    ref.packed = False           # (both forms' kernels are loaded before memory runs short)
+    ref.step(2.4, sr.SR_RK_FIXED)
+    ref.close()
+    ref = sr.Flow(lat, mesh, 3.0, prec)
+    ref.step(2.5, sr.SR_RK_FIXED)
+    exp = [x.cpu() for x in ref.get_state()]
+    ref.close()
+    fl = sr.Flow(lat, mesh, 3.0, prec)
+    part = (8 * fl.n_gamma + 2 * mib - 1) // (2 * mib) * 2 * mib
+    spare = 40 * mib if mixed else 140 * mib       # less than the packed state gives back
+
+    def hog(free):
+        gc.collect()
+        torch.cuda.empty_cache()
+        return torch.empty(torch.cuda.mem_get_info()[0] - free, dtype=torch.uint8, device="cuda")
+
+    h = hog(4 * part)
+    try:
+        with pytest.raises(sr.SrError):
+            fl.step(2.5, sr.SR_RK_FIXED)
+    finally:
+        del h
+    assert fl.packed
+    h = hog(9 * part - spare)
+    try:
+        fl.step(2.5, sr.SR_RK_FIXED)
+    finally:
+        del h
+        torch.cuda.empty_cache()
+    assert not fl.packed
+    for x, y in zip(fl.get_state(), exp):
+        assert _rel(x.cpu(), y) <= (1e-5 if mixed else 1e-12)
+    fl.close()
