@@ -179,8 +179,8 @@ def _algorithmic_flops(counts: np.ndarray, N: int, Ns: int, nc: int, P: int, npr
     equations (an FMA = 2 flop).  Per stored triple (s, t, u) and integration node: every vertex row
     the equations need is interpolated over all irreducible sites and components; one of the three
     frequency arguments of every row is a mesh frequency, so an interpolated value is 4 corners =
-    4 FMA = 8 flop (node weights ride on corner weights).  s and u channels: two rows and one FMA per
-    value (products of eigenvalues).  t channel: two rows, two on-site rows (n_c values each), the
+    4 FMA = 8 flop (node weights ride on corner weights).  s and u channels: two rows and their product
+    per site, 4 FMA (SU2) or 16 (XYZ).  t channel: two rows, two on-site rows (n_c values each), the
     on-site terms (two FMA per value) and the lattice sum as one FMA per distinct product of table
     rows.  TRI (n_c = 16, or 8 with a graded vertex): s / u products n_c x 16 (8) FMA per site, the two
     on-site terms 4 (2) FMA each per value, the lattice sum 64 (16) FMA per pair of sites at most."""
@@ -191,7 +191,7 @@ def _algorithmic_flops(counts: np.ndarray, N: int, Ns: int, nc: int, P: int, npr
         lat_flop = 2 * (16 if graded else 64) * min(P, Ns * Ns)
     else:
         m, row = nc, Ns * nc
-        prod, onsite, lat_flop = 2 * row, 4 * row, 2 * nprod
+        prod, onsite, lat_flop = {2: 8, 4: 32}[nc] * Ns, 4 * row, 2 * nprod
     per_s = 2 * row * 8 + prod
     per_u = per_s
     per_t = (2 * row + 2 * m) * 8 + lat_flop + onsite

@@ -1671,7 +1671,7 @@ static void launch_gamma_tri(sr_flow* f, const double* G_s, const float* Gf_s, d
             if (f->td_graded) trid::k_tri_pack<double, true><<<pblocks, 128, 0, st>>>(g, f->td, G_s, f->Pd.p, f->td_flag);
             else trid::k_tri_pack<double, false><<<pblocks, 128, 0, st>>>(g, f->td, G_s, f->Pd.p, nullptr);
             f->tdd.fn<<<blocks, f->tdd.threads, f->tdd.smem, st>>>(g, tb, f->td, f->w.p, f->Pd.p, f->nx.p, f->nW.p, f->ncount.p,
-                                                                   dG_o, pb, use, 0);
+                                                                   dG_o, pb, use);
         } else {
             if (f->td_graded) {
                 trid::k_tri_pack<float, true><<<pblocks, 128, 0, st>>>(g, f->td, G_s, f->Pf.p, f->td_flag);
@@ -1680,7 +1680,7 @@ static void launch_gamma_tri(sr_flow* f, const double* G_s, const float* Gf_s, d
                 trid::k_tri_pack<float, false><<<pblocks, 128, 0, st>>>(g, f->td, G_s, f->Pf.p, nullptr);
             }
             f->tdf.fn<<<blocks, f->tdf.threads, f->tdf.smem, st>>>(g, tb, f->td, f->w.p, f->Pf.p, f->nx.p, f->nW.p, f->ncount.p,
-                                                                   dG_o, pb, use, 0);
+                                                                   dG_o, pb, use);
         }
         if (!f->td_graded) return;
     }
@@ -1771,10 +1771,8 @@ static sr_status run_rhs(sr_flow* f, double lam, const double* gam_s, const doub
         if (g.nc == 2 && f->dense && f->use_tc)
             k_gamma_rhs_f32_tc<<<std::min(blocks, f->tc_grid), kThreads, f->smem_tc, f->stream>>>(g, tb, Gf_s, Gs, f->nxf.p, f->nWf.p, f->ncount.p, dG_o,
                                                                             f->flag.p + 1, (long)pb * g.N, (long)pe * g.N);
-        else if (g.nc == 2 && f->dense)
-            k_gamma_rhs_f32<2, true><<<blocks, kThreads, f->smem_rhs, f->stream>>>(g, tb, Gf_s, Gs, f->nxf.p, f->nWf.p, f->ncount.p, dG_o, pb);
         else if (g.nc == 2)
-            k_gamma_rhs_f32<2, false><<<blocks, kThreads, f->smem_rhs, f->stream>>>(g, tb, Gf_s, Gs, f->nxf.p, f->nWf.p, f->ncount.p, dG_o, pb);
+            k_gamma_rhs_f32<2, true><<<blocks, kThreads, f->smem_rhs, f->stream>>>(g, tb, Gf_s, Gs, f->nxf.p, f->nWf.p, f->ncount.p, dG_o, pb);
         else
             k_gamma_rhs_f32<4, false><<<blocks, kThreads, f->smem_rhs, f->stream>>>(g, tb, Gf_s, Gs, f->nxf.p, f->nWf.p, f->ncount.p, dG_o, pb);
     }
@@ -2093,7 +2091,7 @@ static sr_status flow_create(const sr_lattice* lat, int n_freq, const double* fr
             f->chi_counter = (int*)(base + o_cnt);   // zero between launches
             CK(f->chi_part.alloc(chik::part_doubles(g.Ns, g.nc)));
             const size_t sm = sizeof(double) * 2 * g.Ns * g.nc * chik::groups(g.Ns * g.nc);
-            if (sm > 32 * 1024) CK(ensure_smem(g.nc == 2 ? (const void*)chik::k_chi_sum<2> : (const void*)chik::k_chi_sum<4>, sm));
+            if (sm > 24 * 1024) CK(ensure_smem(g.nc == 2 ? (const void*)chik::k_chi_sum<2> : (const void*)chik::k_chi_sum<4>, sm));
         }
     }
     if (lat->nc == 16) {
@@ -2268,7 +2266,6 @@ static sr_status flow_create(const sr_lattice* lat, int n_freq, const double* fr
         CK(ensure_smem((const void*)k_gamma_rhs<double, 4>, f->smem_rhs));
     } else {
         CK(ensure_smem((const void*)k_gamma_rhs_f32<2, true>, f->smem_rhs));
-        CK(ensure_smem((const void*)k_gamma_rhs_f32<2, false>, f->smem_rhs));
         CK(ensure_smem((const void*)k_gamma_rhs_f32<4, false>, f->smem_rhs));
         if (tc_ok) {
             // persistent grid: resident CTAs per SM limited by the kernel's resources and by
@@ -3556,7 +3553,6 @@ extern "C" sr_status sr_batch_create(int n, sr_flow* const* flows, sr_batch** ou
         B.P = f->Pf.p;
         B.flow = f;
         B.copy_f32 = f->td_on ? 0 : 1;
-        if (kind[k] == 0) B.qc = pairk::qrows<float>();
         unit += (long)f->g.npair * f->g.N;
         b->inst.push_back(B);
         b->inst_smem.push_back(f->smem_rhs);

@@ -264,13 +264,13 @@ __device__ __forceinline__ void su_acc(const R* a, const R* b, R* o) {
 }
 
 // dGamma/dLambda of one stored triple per CTA.  P: packed state (plain rows, then exchanged rows).
-// use: nullptr, or the flag of k_tri_pack with the value this form serves.
+// use: nullptr, or the flag of k_tri_pack (zero: this form serves the state).
 template <typename R, bool GR, int TM, int TN, int NT, int MAXT, int MINB>
 __global__ void __launch_bounds__(MAXT, MINB)
 k_gamma_rhs_trid(Geo g, Tabs tb, Tab td, const double* __restrict__ w, const R* __restrict__ P, const double* __restrict__ nx,
                  const double* __restrict__ nW, const int* __restrict__ ncount, double* __restrict__ dG, int p0,
-                 const int* __restrict__ use, int use_value) {
-    if (use && (*use != 0) != (use_value != 0)) return;
+                 const int* __restrict__ use) {
+    if (use && *use != 0) return;   // the general kernel serves this state
     constexpr int NCm = ncomp<GR>(), NM = nmu<GR>(), QB = qblock<R>();
     extern __shared__ __align__(16) unsigned char smem[];
     const int tid = threadIdx.x, nth = blockDim.x, Ns = g.Ns;
@@ -605,7 +605,7 @@ __global__ void k_shadow_if(long n, const double* __restrict__ G, float* __restr
 
 template <typename R>
 using Kernel = void (*)(Geo, Tabs, Tab, const double*, const R*, const double*, const double*, const int*, double*, int,
-                        const int*, int);
+                        const int*);
 
 template <typename R>
 struct Variant {
@@ -640,8 +640,8 @@ struct Choice {
     size_t smem = 0;
 };
 
-// The first variant that fills at least three warps with tiles, else the last that fits; none when
-// the tiles or the shared memory exceed one CTA.
+// The first variant that fits a CTA and fills at least three warps with tiles; where none fills them
+// (lattices of a few sites), the first that fits; none when the tiles or the shared memory exceed one CTA.
 template <typename R, bool GR>
 inline Choice<R> choose(int N, int Ns, int nk, int n_runs) {
     Choice<R> c;
