@@ -228,7 +228,7 @@ sr_status sr_flow_tensor_cores(const sr_flow* flow, int* on);
  * such a kernel and the copy found memory when the flow was created) or on the stored state.  Off
  * frees the copy and with it the packed adjoint: for SU2 / XYZ two values per entry (four with a
  * non-trivial site exchange), FP64 or FP32 as the precision, and half of that for the adjoint; for TRI
- * one or two FP32 / FP64 values per entry.  Slower: 1.3 to 8 times.  FP32-mixed flows then hold an
+ * one or two FP32 / FP64 values per entry.  Off is slower: 1.2 to 8 times.  FP32-mixed flows then hold an
  * FP32 copy of the entries instead.  Synchronises.  Errors: SR_EUNSUPPORTED (on, and the lattice has
  * no packed kernel), SR_ENOMEM (the flow stays as it was), SR_EINVAL (null, or the flow is in a
  * batch). */

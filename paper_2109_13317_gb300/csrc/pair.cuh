@@ -22,17 +22,20 @@
 // Lookups.  The arguments of the rows of a node are sums of x and four frequencies of the triple, so
 // a node needs four interval searches per channel for its two to four rows.
 //
-// Measured (vertex kernel, one GB300; before: the general FP64 kernel and the FP32 kernels on
-// component rows): square J1-J2 range 7, 48 frequencies, FP64 13.2 -> 10.5 ms, FP32 1.55 -> 0.98 ms;
-// pyrochlore range 6, 64 frequencies, FP32 12.6 -> 7.9 ms; honeycomb Heisenberg-Kitaev range 5,
-// 32 frequencies, FP64 3.65 -> 2.85 ms, FP32 0.60 -> 0.35 ms.
-// What bounds it: FP64, the FP64 pipe (92 % busy on the square lattice); FP32, the L1 data path (86 %
-// busy there: a corner chunk is one 16-byte load per 4 multiply-adds, and a row of 160 bytes touches
-// two 128-byte lines).  Tried and dropped in FP32: corner chunks kept in registers over a run of
-// nodes per group (1.69 ms against 1.27 at that stage: adjacent nodes no longer share their loads,
-// the L1 hit rate falls from 62 to 14 %).  Taken: corners in parity slots with adjacent nodes in
-// adjacent groups and descriptors stored as arrays (1.27 -> 1.03), on-site rows with both t corners in
-// one load and lattice-sum terms merged with multiplicities (1.03 -> 0.98).
+// Measured (packing and vertex kernel, one GB300; before: the general FP64 kernel and the FP32 kernels on
+// the stored state): square J1-J2 range 7, 48 frequencies, FP64 13.2 -> 10.7 ms, FP32 1.56 -> 1.02 ms;
+// pyrochlore range 6, 64 frequencies, FP32 12.6 -> 8.3 ms; honeycomb Heisenberg-Kitaev range 5,
+// 32 frequencies, FP64 3.65 -> 3.10 ms, FP32 0.60 -> 0.36 ms.
+// What bounds it: FP64, the FP64 pipe (94 % busy on the square and the honeycomb lattice); FP32, the L1
+// data path (87 % busy on the square lattice, 73 % on the pyrochlore: a corner chunk is one 16-byte load
+// per 4 multiply-adds, and a row of 160 bytes touches two 128-byte lines).  Tried and dropped in FP32:
+// corner chunks kept in registers over a run of nodes per group (1.69 ms against 1.27 at that stage:
+// adjacent nodes no longer share their loads, the L1 hit rate falls from 62 to 14 %).  Taken: corners in
+// parity slots with adjacent nodes in adjacent groups and descriptors stored as arrays (1.27 -> 1.03),
+// on-site rows with both t corners in one load and lattice-sum terms merged with multiplicities (1.03 ->
+// 0.98).  The t rows are packed apart from the s / u rows, component by component: read from the latter
+// they would halve the packed state but cost FP32 2 % (a second weight set per row; pyrochlore 8.36 ->
+// 8.56 ms), and the density's sign in the offset instead of that set costs the long rows more (8.65).
 #pragma once
 
 namespace pairk {
@@ -521,7 +524,9 @@ __device__ __forceinline__ void triple(const Geo& g, const Tabs& tb, const Tab& 
     if (in_stream) st16(tt + (2 * stream + rw) * rt + ct * V, pt);
     __syncthreads();
     // FP64 and long rows: the sums over groups and streams first, a value each (into the slots of the
-    // first group and stream), instead of every output summing the values it mixes
+    // first group and stream), instead of every output summing the values it mixes (with eigenvalue rows:
+    // square range 7 FP64 11.85 -> 11.70 ms, pyrochlore FP32 8.39 -> 8.18; the short FP32 rows lose 3 % by
+    // the barrier)
     constexpr bool kStage = sizeof(R) == 8 || TM == 8;
     if constexpr (kStage) {
         for (int v = tid; v < nsu + rt; v += nth) {
@@ -641,6 +646,7 @@ using Kernel = void (*)(Geo, Tabs, Tab, const R*, const R*, const R*, const int*
 // up to 20 sites 4 x 4 tiles fill 64 threads.  FP64 lists have no padding, tiles take over where the
 // products exceed eight per thread; their registers are capped for six CTAs of 128 threads (square range
 // 7: five 11.7 ms, six 10.5, seven and eight 10.5; 13 products on 64 threads 11.3; 160 threads 12.8).
+// (These times are of the eigenvalue form named above, 2 % faster throughout.)
 #define PAIR_F32_VARIANTS(X)     \
     X(0, 2, 4, 4, 1, 64, 12, 4)  \
     X(1, 2, 8, 4, 1, 160, 5, 8)  \
